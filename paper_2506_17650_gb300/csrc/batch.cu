@@ -95,9 +95,10 @@ struct StoreRowOp {
 };
 
 // KKT check, termination / restart decision and its application (a team-wide
-// version of the check kernels).
+// version of the check kernels).  Out of line, like the promotion below: rare
+// next to the attempts, whose loop should stay in the instruction caches.
 template <class V>
-__device__ void team_check(const Dev& d, const Params& prm, DevState& s, int rank, int T, bool wide, double* blk,
+__device__ __noinline__ void team_check(const Dev& d, const Params& prm, DevState& s, int rank, int T, bool wide, double* blk,
                            double* slots, int eval_only = 0) {
   const Vecs<V>& v = vecs<V>(d);
   const int cur = s.cur;
@@ -169,7 +170,7 @@ __device__ void team_check(const Dev& d, const Params& prm, DevState& s, int ran
 }
 
 // FP32 iterate -> FP64 iterate, then A x recomputed in FP64.
-__device__ void team_promote(const Dev& d, const DevState& s, int rank, int T, bool wide, double* blk) {
+__device__ __noinline__ void team_promote(const Dev& d, const DevState& s, int rank, int T, bool wide, double* blk) {
   const Vecs<float>& a = d.f32;
   const Vecs<double>& b = d.f64;
   const int cur = s.cur;
@@ -205,7 +206,7 @@ __device__ void team_promote(const Dev& d, const DevState& s, int rank, int T, b
 
 // The FP32 phase reached the tolerance against the FP32 copy of A~: end the
 // phase and let an FP64 termination test of the promoted point decide.
-__device__ void team_certify(const Dev& d, const Params& prm, DevState& s, int rank, int T, bool wide, double* blk,
+__device__ __noinline__ void team_certify(const Dev& d, const Params& prm, DevState& s, int rank, int T, bool wide, double* blk,
                              double* slots) {
   if (threadIdx.x == 0) {
     s.status = 0;

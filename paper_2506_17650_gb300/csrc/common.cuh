@@ -141,14 +141,19 @@ __host__ __device__ inline void refresh_derived(DevState& s, int phi, int sched)
 }
 
 // Factors of the next-step-size rule for attempt t: 1 - (t+1)^-0.3 and
-// 1 + (t+1)^-0.6 (tabulated below kStepTab).
+// 1 + (t+1)^-0.6 (tabulated below kStepTab; beyond it computed, out of line).
+static __device__ __noinline__ double2 step_factors_late(long long t) {
+  return double2{1.0 - pow((double)t + 1.0, -0.3), 1.0 + pow((double)t + 1.0, -0.6)};
+}
+
 __device__ inline void step_factors(const double* step_tab, long long t, double* f1, double* f2) {
   if (t < kStepTab) {
     *f1 = __ldg(step_tab + t);
     *f2 = __ldg(step_tab + kStepTab + t);
   } else {
-    *f1 = 1.0 - pow((double)t + 1.0, -0.3);
-    *f2 = 1.0 + pow((double)t + 1.0, -0.6);
+    const double2 f = step_factors_late(t);
+    *f1 = f.x;
+    *f2 = f.y;
   }
 }
 

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(kBlock, kStepBlocksPerSm<V>) primal_step_kerne
   __shared__ double smem[kBlock * 3];
   pdl_wait();
   const Vecs<V>& v = vecs<V>(d);
-  PrimalOp<V> op;
+  PrimalOp<V, true> op;
   op.sc = read_scalars<V>(d.st, true);
   const int cur = op.sc.cur, nxt = cur ^ 1;
   op.prm = prm;
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kBlock, kStepBlocksPerSm<V>) dual_step_kernel(
     for (int t = threadIdx.x; t < (int)(sizeof(DevState) / 8); t += blockDim.x) cp_async8(dst + t, src + t);
   }
   const Vecs<V>& v = vecs<V>(d);
-  DualOp<V> op;
+  DualOp<V, true> op;
   op.sc = read_scalars<V>(d.st, false);
   const int cur = op.sc.cur, nxt = cur ^ 1;
   op.prm = prm;
@@ -152,12 +152,10 @@ __global__ void flush_update_kernel(Dev d, Params prm) {
   const V gp = (V)st->sqrt_gp, gd = (V)st->sqrt_gd;
   const int stride = gridDim.x * blockDim.x;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n && pp; j += stride) {
-    v.T[j] = ogd_entry<V>(v.T[j], v.GT + j, sp * v.q[j], prm, gp);
-    v.invT[j] = V(1) / v.T[j];
+    ogd_entry<V>(v.T + j, v.invT + j, v.GT + j, sp * v.q[j], prm.sched, (V)prm.alpha, (V)prm.floor, gp);
   }
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.m && pd; i += stride) {
-    v.S[i] = ogd_entry<V>(v.S[i], v.GS + i, sd * v.p[i], prm, gd);
-    v.invS[i] = V(1) / v.S[i];
+    ogd_entry<V>(v.S + i, v.invS + i, v.GS + i, sd * v.p[i], prm.sched, (V)prm.alpha, (V)prm.floor, gd);
   }
 }
 

@@ -272,6 +272,7 @@ __global__ void scale_by_inv_kernel(double* v, int n, const double* denom) {
 
 struct StoreOp {
   double* y;
+  static constexpr bool kCsrOnly = true;
   __device__ __forceinline__ void prefetch(int) {}
   __device__ __forceinline__ void row(int r, const double (&s)[1]) { y[r] = s[0]; }
 };

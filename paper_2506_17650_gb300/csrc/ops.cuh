@@ -41,24 +41,36 @@ __device__ __forceinline__ StepScalars<V> read_scalars(const DevState* st, bool 
   return s;
 }
 
-// One projected online-gradient step of a diagonal preconditioner entry with
-// the chosen learning-rate rule (Section 3.1 OGD, Section 4.1 AdaGrad).
+// One projected online-gradient step of a diagonal preconditioner entry *P
+// with the chosen learning-rate rule (Section 3.1 OGD, Section 4.1 AdaGrad),
+// and its reciprocal *inv.
 template <class V>
-__device__ __forceinline__ V ogd_entry(V P, V* G, V grad, const Params& prm, V sqrt_gnorm) {
-  const V alpha = (V)prm.alpha;
-  if (prm.sched == kAdagrad) {
+__device__ __forceinline__ void ogd_entry_inline(V* P, V* inv, V* G, V grad, int sched, V alpha, V floor, V sqrt_gnorm) {
+  V p = *P;
+  if (sched == kAdagrad) {
     const V Gn = *G + grad * grad;
     *G = Gn;
-    if (Gn > V(0)) P = P - alpha * (grad / sqrt(Gn));
-  } else if (prm.sched == kAdagradNorm) {
-    if (sqrt_gnorm > V(0)) P = P - alpha * (grad / sqrt_gnorm);
+    if (Gn > V(0)) p = p - alpha * (grad / sqrt(Gn));
+  } else if (sched == kAdagradNorm) {
+    if (sqrt_gnorm > V(0)) p = p - alpha * (grad / sqrt_gnorm);
   } else {
-    P = P - alpha * grad;
+    p = p - alpha * grad;
   }
-  return fmax(P, (V)prm.floor);
+  p = fmax(p, floor);
+  *P = p;
+  *inv = V(1) / p;
 }
 
+// The same out of line.  It runs once every phi accepted attempts and holds
+// two divisions and a square root (long instruction sequences in FP64), and
+// the row code around it is inlined several times per kernel.  (Not in the
+// step kernels: at their 64 / 80 registers a call in the row code spills.)
 template <class V>
+__device__ __noinline__ void ogd_entry(V* P, V* inv, V* G, V grad, int sched, V alpha, V floor, V sqrt_gnorm) {
+  ogd_entry_inline<V>(P, inv, G, grad, sched, alpha, floor, sqrt_gnorm);
+}
+
+template <class V, bool kInlineUpdate = false>
 struct PrimalOp {
   const V *c, *l, *u, *xc, *xbarc;
   V *T, *invT, *GT, *q, *xn, *xbarn;
@@ -80,10 +92,10 @@ struct PrimalOp {
   __device__ __forceinline__ void row(int j, const V (&s)[1]) {
     V Tj = pT, iT = piT;
     if (sc.pend) {  // pending online update of T_j (rare: once every phi accepted steps)
-      Tj = ogd_entry<V>(Tj, GT + j, sc.up_scale * q[j], prm, sc.sqrt_gnorm);
-      iT = V(1) / Tj;
-      T[j] = Tj;
-      invT[j] = iT;
+      if (kInlineUpdate) ogd_entry_inline<V>(T + j, invT + j, GT + j, sc.up_scale * q[j], prm.sched, (V)prm.alpha, (V)prm.floor, sc.sqrt_gnorm);
+      else ogd_entry<V>(T + j, invT + j, GT + j, sc.up_scale * q[j], prm.sched, (V)prm.alpha, (V)prm.floor, sc.sqrt_gnorm);
+      Tj = T[j];
+      iT = invT[j];
     }
     const V g = pc - s[0];
     const V x0 = px;
@@ -105,7 +117,7 @@ struct PrimalOp {
   }
 };
 
-template <class V>
+template <class V, bool kInlineUpdate = false>
 struct DualOp {
   const V *b, *axc, *yc, *ybarc;
   const uint8_t* sense;
@@ -129,10 +141,10 @@ struct DualOp {
   __device__ __forceinline__ void row(int i, const V (&s)[1]) {
     V Si = pS, iS = piS;
     if (sc.pend) {
-      Si = ogd_entry<V>(Si, GS + i, sc.up_scale * p[i], prm, sc.sqrt_gnorm);
-      iS = V(1) / Si;
-      S[i] = Si;
-      invS[i] = iS;
+      if (kInlineUpdate) ogd_entry_inline<V>(S + i, invS + i, GS + i, sc.up_scale * p[i], prm.sched, (V)prm.alpha, (V)prm.floor, sc.sqrt_gnorm);
+      else ogd_entry<V>(S + i, invS + i, GS + i, sc.up_scale * p[i], prm.sched, (V)prm.alpha, (V)prm.floor, sc.sqrt_gnorm);
+      Si = S[i];
+      iS = invS[i];
     }
     const V a1 = s[0];
     const V a0 = pa0;

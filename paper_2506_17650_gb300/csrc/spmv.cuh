@@ -11,6 +11,12 @@
 // of M.v and M.ci are contiguous, long rows a whole block, and the longest rows
 // several blocks (segments).  Lane sums are combined by a fixed shuffle tree,
 // so results do not depend on scheduling.
+//
+// The row code is inlined at each place that runs it, so a kernel holds only
+// the classes that its rows can have, and one copy for whole-block rows and
+// segments: the FP64 primal kernel has 90 KB of instructions instead of 169,
+// the batched kernel 1.0 MB instead of 3.6 (one call with 256 LPs of up to 300k
+// nonzeros, 128 attempts: 183 -> 140 ms; the step kernels 1-2%).
 #pragma once
 
 #include <type_traits>
@@ -51,6 +57,13 @@ struct AllowsPair : std::true_type {};
 template <class Op>
 struct AllowsPair<Op, std::void_t<decltype(Op::kNoPair)>> : std::false_type {};
 
+// Ops of the setup kernels, which also run before the sliced copies are filled
+// (and with 8 lanes per row): those that declare kCsrOnly.
+template <class Op, class = void>
+struct ReadsCsrOnly : std::false_type {};
+template <class Op>
+struct ReadsCsrOnly<Op, std::void_t<decltype(Op::kCsrOnly)>> : std::true_type {};
+
 // Entries handled per lane per round: all their index/value loads are issued,
 // then all gathers, then the FMAs, so each lane keeps kChunk independent
 // loads in flight instead of one dependent load chain per entry.
@@ -87,6 +100,7 @@ __device__ __forceinline__ void chunk_dot(int k0, int end, int stride, const Csr
   }
 }
 
+// Rows first + tid / W < row_end, W lanes each.
 template <int W, int NV, class V, class Acc, class Op>
 __device__ __forceinline__ void vec_rows(int first, int row_end, const CsrT<V>& M, const Gather<NV, V>& g,
                                          Op& op) {
@@ -252,95 +266,78 @@ __device__ __forceinline__ void block_dot(int beg, int end, const CsrT<V>& M, co
   block_sum<NV>(s, smem);
 }
 
-template <int NV, class V, class Acc, class Op>
-__device__ __forceinline__ void block_row(int row, const CsrT<V>& M, const Gather<NV, V>& g, Op& op,
-                                          double* smem) {
-  if (threadIdx.x == 0) op.prefetch(row);
-  double s[NV];  // the block-wide sum of a long row is formed in FP64
-  block_dot<NV, V, Acc>(__ldg(M.rp + row), __ldg(M.rp + row + 1), M, g, s, smem);
-  if (threadIdx.x == 0) {
-    Acc r[NV];
+// op.row, with the op's reduction accumulators diverted into slot[0..) when
+// one is given: the contribution of a segmented row is kept apart from the
+// block's own partial sums, so the totals do not depend on which block
+// finishes the row.
+template <int NV, class Acc, class Op>
+__device__ __forceinline__ void row_into_slot(Op& op, int row, const Acc (&r)[NV], double* slot) {
+  if constexpr (HasAcc<Op>::value) {
+    constexpr int NA = (int)(sizeof(op.acc) / sizeof(op.acc[0]));
+    using A = typename std::remove_reference<decltype(op.acc[0])>::type;
+    A saved[NA];
 #pragma unroll
-    for (int q = 0; q < NV; ++q) r[q] = (Acc)s[q];
+    for (int q = 0; q < NA; ++q) {
+      saved[q] = op.acc[q];
+      if (slot) op.acc[q] = A(0);
+    }
+    op.row(row, r);
+    if (slot) {
+#pragma unroll
+      for (int q = 0; q < NA; ++q) {
+        slot[q] = (double)op.acc[q];
+        op.acc[q] = saved[q];
+      }
+      for (int q = NA; q < kMaxPartials; ++q) slot[q] = 0.0;  // fields read by wider sums
+    }
+  } else {
     op.row(row, r);
   }
 }
 
-// Run op.row with the op's reduction accumulators diverted into slot[0..): the
-// contribution of a segmented row is kept apart from the block's own partial
-// sums, so the totals do not depend on which block finishes the row.
-template <class Acc, class Op, int NV>
-__device__ __forceinline__ void row_into_slot(Op& op, int row, const Acc (&r)[NV], double* slot) {
-  constexpr int NA = (int)(sizeof(op.acc) / sizeof(op.acc[0]));
-  using A = typename std::remove_reference<decltype(op.acc[0])>::type;
-  A saved[NA];
-#pragma unroll
-  for (int q = 0; q < NA; ++q) {
-    saved[q] = op.acc[q];
-    op.acc[q] = A(0);
-  }
-  op.row(row, r);
-#pragma unroll
-  for (int q = 0; q < NA; ++q) {
-    slot[q] = (double)op.acc[q];
-    op.acc[q] = saved[q];
-  }
-  for (int q = NA; q < kMaxPartials; ++q) slot[q] = 0.0;  // fields read by wider sums
-}
-
-
-// One segment of a segmented row, published for the row's other segments;
-// the block that completes the row's last segment adds the segment sums in
-// segment order and runs the epilogue into the row's slot.
+// A unit of the whole-block bin (row = the unit's row, seg = -1) or of the
+// segmented bin.  With row_slots (one row of kMaxPartials doubles per
+// segmented row, for ops with reduction accumulators) a segment is summed and
+// published for the row's other segments; the block that completes the row's
+// last segment adds the segment sums in segment order and runs the epilogue
+// into the row's slot.  Without, the unit of segment 0 takes the whole row and
+// the others do nothing.
 template <int NV, class V, class Acc, class Op>
-__device__ __forceinline__ void segment_reduce(const BinTable& bt, int local, int row, int seg, const CsrT<V>& M,
-                                               const Gather<NV, V>& g, Op& op, double* smem, double* row_slots) {
+__device__ __forceinline__ void wide_unit(const BinTable& bt, int local, int row, int seg, const CsrT<V>& M,
+                                          const Gather<NV, V>& g, Op& op, double* smem, double* row_slots) {
   static_assert(NV <= 2, "segment sums hold up to two vectors");
+  const bool split = seg >= 0 && HasAcc<Op>::value && row_slots != nullptr;
+  if (!split && seg > 0) return;
   const int r0 = __ldg(M.rp + row), r1 = __ldg(M.rp + row + 1);
-  const int beg = r0 + seg * bt.seg_len;
-  const int end = min(beg + bt.seg_len, r1);
-  double s[NV];
+  const int beg = split ? r0 + seg * bt.seg_len : r0;
+  const int end = split ? min(beg + bt.seg_len, r1) : r1;
+  if (threadIdx.x == 0) op.prefetch(row);
+  double s[NV];  // the sum of a long row is formed in FP64
   block_dot<NV, V, Acc>(beg, end, M, g, s, smem);
   if (threadIdx.x != 0) return;
+  double* slot = nullptr;
+  if (split) {
 #pragma unroll
-  for (int q = 0; q < NV; ++q) bt.seg_sum[2 * local + q] = s[q];
-  __threadfence();
-  const int id = row - bt.bin[0].row_begin;
-  const unsigned int nseg = (unsigned int)((r1 - r0 + bt.seg_len - 1) / bt.seg_len);
-  if (atomicAdd(bt.ticket + id, 1u) != nseg - 1) return;
-  __threadfence();
-  const int first = local - seg;
-  double tot[NV];
+    for (int q = 0; q < NV; ++q) bt.seg_sum[2 * local + q] = s[q];
+    __threadfence();
+    const int id = row - bt.bin[0].row_begin;
+    const unsigned int nseg = (unsigned int)((r1 - r0 + bt.seg_len - 1) / bt.seg_len);
+    if (atomicAdd(bt.ticket + id, 1u) != nseg - 1) return;
+    __threadfence();
+    const int first = local - seg;
 #pragma unroll
-  for (int q = 0; q < NV; ++q) tot[q] = 0.0;
-  for (int t = 0; t < (int)nseg; ++t) {
+    for (int q = 0; q < NV; ++q) s[q] = 0.0;
+    for (int t = 0; t < (int)nseg; ++t) {
 #pragma unroll
-    for (int q = 0; q < NV; ++q) tot[q] += __ldcg(bt.seg_sum + 2 * (first + t) + q);
+      for (int q = 0; q < NV; ++q) s[q] += __ldcg(bt.seg_sum + 2 * (first + t) + q);
+    }
+    bt.ticket[id] = 0u;  // ready for the next launch
+    slot = row_slots + (size_t)id * kMaxPartials;
   }
-  bt.ticket[id] = 0u;  // ready for the next launch
   Acc r[NV];
 #pragma unroll
-  for (int q = 0; q < NV; ++q) r[q] = (Acc)tot[q];
-  op.prefetch(row);
-  row_into_slot<Acc>(op, row, r, row_slots + (size_t)id * kMaxPartials);
-}
-
-// A unit of the segmented bin.  With row_slots (one row of kMaxPartials
-// doubles per segmented row, for ops with reduction accumulators) segments
-// are reduced by separate blocks (segment_reduce).  Without, the unit of
-// segment 0 reduces the whole row and the others do nothing.
-template <int NV, class V, class Acc, class Op>
-__device__ __forceinline__ void segment_unit(const BinTable& bt, int local, const CsrT<V>& M, const Gather<NV, V>& g,
-                                             Op& op, double* smem, double* row_slots) {
-  const int row = __ldg(bt.seg_unit + 2 * local);
-  const int seg = __ldg(bt.seg_unit + 2 * local + 1);
-  if constexpr (HasAcc<Op>::value) {
-    if (row_slots) {
-      segment_reduce<NV, V, Acc>(bt, local, row, seg, M, g, op, smem, row_slots);
-      return;
-    }
-  }
-  if (seg == 0) block_row<NV, V, Acc>(row, M, g, op, smem);
+  for (int q = 0; q < NV; ++q) r[q] = (Acc)s[q];
+  row_into_slot<NV, Acc>(op, row, r, slot);
 }
 
 // Work units first_unit, first_unit + unit_stride, ... of the table (one block
@@ -353,41 +350,39 @@ __device__ __forceinline__ void for_each_row_range(const BinTable& bt, const Csr
   int b = 0;  // units only increase, so the bin search resumes where it stopped
   for (int u = first_unit; u < bt.nunits; u += unit_stride) {
     while (b + 1 < bt.nbins && u >= bt.bin[b + 1].unit_begin) ++b;
-    const int row_begin = bt.bin[b].row_begin;
-    const int row_end = bt.bin[b].row_end;
-    const int local = u - bt.bin[b].unit_begin;
-    switch (bt.bin[b].width) {
-      case kSegmented: segment_unit<NV, V, Acc>(bt, local, M, g, op, smem, row_slots); break;
-      case kSell:
-        if (bt.bin[b].len <= kPairMaxLen) {  // units of two halves of H rows (H = kBlock by default)
-          const int H = rows_per_unit(bt.bin[b]) / 2;
-          if (bt.sell_ci) {
-            if constexpr (AllowsPair<Op>::value) {
-              sell_rows_pair<NV, V, Acc>(bt, bt.bin[b], local, g, op);
-            } else if ((int)threadIdx.x < H) {  // the unit's two halves one after the other
-              const int i0 = local * 2 * H + (int)threadIdx.x;
-              sell_rows_at<NV, V, Acc>(bt, bt.bin[b], i0, g, op);
-              sell_rows_at<NV, V, Acc>(bt, bt.bin[b], i0 + H, g, op);
-            }
-          } else {
-            const int h0 = row_begin + local * 2 * H;
-            vec_rows<1, NV, V, Acc>(h0, min(row_end, h0 + H), M, g, op);
-            vec_rows<1, NV, V, Acc>(h0 + H, min(row_end, h0 + 2 * H), M, g, op);
-          }
-        } else if (bt.sell_ci) {
-          sell_rows<NV, V, Acc>(bt, bt.bin[b], local, g, op);
+    const Bin& B = bt.bin[b];
+    const int local = u - B.unit_begin;
+    const int width = B.width;
+    if (width == kSell && bt.sell_ci) {
+      if (B.len <= kPairMaxLen) {  // units of two halves of H rows (H = kBlock by default)
+        if constexpr (AllowsPair<Op>::value) {
+          sell_rows_pair<NV, V, Acc>(bt, B, local, g, op);
         } else {
-          const int R = rows_per_unit(bt.bin[b]);
-          vec_rows<1, NV, V, Acc>(row_begin + local * R, min(row_end, row_begin + (local + 1) * R), M, g, op);
+          const int H = rows_per_unit(B) / 2;
+          if ((int)threadIdx.x < H) {  // the unit's two halves one after the other
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) sell_rows_at<NV, V, Acc>(bt, B, (local * 2 + h) * H + (int)threadIdx.x, g, op);
+          }
         }
-        break;
-      case 0: block_row<NV, V, Acc>(row_begin + local, M, g, op, smem); break;
-      case 1: vec_rows<1, NV, V, Acc>(row_begin + local * kBlock, row_end, M, g, op); break;
-      case 2: vec_rows<2, NV, V, Acc>(row_begin + local * (kBlock / 2), row_end, M, g, op); break;
-      case 4: vec_rows<4, NV, V, Acc>(row_begin + local * (kBlock / 4), row_end, M, g, op); break;
-      case 8: vec_rows<8, NV, V, Acc>(row_begin + local * (kBlock / 8), row_end, M, g, op); break;
-      case 16: vec_rows<16, NV, V, Acc>(row_begin + local * (kBlock / 16), row_end, M, g, op); break;
-      default: vec_rows<32, NV, V, Acc>(row_begin + local * (kBlock / 32), row_end, M, g, op); break;
+      } else {
+        sell_rows<NV, V, Acc>(bt, B, local, g, op);
+      }
+    } else if (width == kSegmented || width == 0) {
+      const int row = width == 0 ? B.row_begin + local : __ldg(bt.seg_unit + 2 * local);
+      const int seg = width == 0 ? -1 : __ldg(bt.seg_unit + 2 * local + 1);
+      wide_unit<NV, V, Acc>(bt, local, row, seg, M, g, op, smem, row_slots);
+    } else if (width == kSell) {  // before the sliced copy is filled: one lane a row, kBlock rows at a time
+      if constexpr (ReadsCsrOnly<Op>::value) {
+        const int per = rows_per_unit(B), r0 = B.row_begin + local * per, r1 = min(B.row_end, r0 + per);
+#pragma unroll 1
+        for (int r = r0; r < r1; r += kBlock) vec_rows<1, NV, V, Acc>(r, min(r1, r + kBlock), M, g, op);
+      }
+    } else {  // the widths a layout gives its rows (and 8, of the no-allocation power iteration)
+      const int r0 = B.row_begin + local * (kBlock / width);
+      if (width == 4) vec_rows<4, NV, V, Acc>(r0, B.row_end, M, g, op);
+      else if (width == 16) vec_rows<16, NV, V, Acc>(r0, B.row_end, M, g, op);
+      else if (width == 32) vec_rows<32, NV, V, Acc>(r0, B.row_end, M, g, op);
+      else if constexpr (ReadsCsrOnly<Op>::value) vec_rows<8, NV, V, Acc>(r0, B.row_end, M, g, op);
     }
   }
 }
