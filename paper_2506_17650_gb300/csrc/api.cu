@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -20,6 +21,7 @@
 #include "common.cuh"
 #include "device_layout.hpp"
 #include "host_layout.hpp"
+#include "resident.hpp"
 
 using namespace lpop;
 
@@ -39,6 +41,7 @@ void set_thread_error(const std::string& msg) { g_last_error = msg; }
 struct lp_problem {
   lp_options opt{};
   int device = 0;
+  int sms = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   Dev d{};
@@ -80,6 +83,14 @@ struct lp_problem {
   long long sell_n[2] = {0, 0};
   RuizSplit ruiz[2] = {};  // how the Ruiz kernels cut the rows of A / A^T
   long long checks_seen = 0;  // KKT checks run by lp_solve since create (for log_every)
+  // resident check periods, FP64 (0) and FP32 (1): the plan's device block,
+  // taken by lp_create and filled by the first lp_solve
+  struct Resident {
+    char* block = nullptr;
+    bool tried = false;
+    bool ok = false;
+    ResPlan plan{};
+  } res[2];
   int* sell_ci[2] = {nullptr, nullptr};
   double* sell_v[2] = {nullptr, nullptr};
   float* sell_v32[2] = {nullptr, nullptr};
@@ -208,10 +219,13 @@ int select_device(lp_problem* p) {
   return LP_OK;
 }
 
-int read_status(lp_problem* p, int* status) {
-  CK(cudaMemcpyAsync(p->h_status, &p->d.st->status, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
+// status (and fault, see DevState) after the stream's work so far
+int read_status(lp_problem* p, int* status, int* fault = nullptr) {
+  static_assert(offsetof(DevState, fault) == offsetof(DevState, status) + sizeof(int), "read together");
+  CK(cudaMemcpyAsync(p->h_status, &p->d.st->status, 2 * sizeof(int), cudaMemcpyDeviceToHost, p->stream));
   CK(cudaStreamSynchronize(p->stream));
-  *status = *p->h_status;
+  *status = p->h_status[0];
+  if (fault) *fault = p->h_status[1];
   return LP_OK;
 }
 
@@ -475,8 +489,8 @@ int upload(lp_problem* p, int m, int n, long long nz, const int64_t* row_ptr, co
     if (!d.step_tab) return set_err(p, LP_ERR_CUDA, std::string("step-size table: ") + cudaGetErrorString(te));
   }
 
-  int sms = 0;
-  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
+  CK(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device));
+  const int sms = p->sms;
   int per_sm_p = 1, per_sm_d = 1, per_sm_p32 = 1, per_sm_d32 = 1;
   row_kernel_blocks_per_sm(&per_sm_p, &per_sm_d, &per_sm_p32, &per_sm_d32);
   d.max_grid = sms * std::max(std::max(per_sm_p, per_sm_d), std::max(per_sm_p32, per_sm_d32));
@@ -538,6 +552,10 @@ int upload(lp_problem* p, int m, int n, long long nz, const int64_t* row_ptr, co
   const int maxg = rows_a > rows_at ? rows_a : rows_at;
   TRY(dalloc(p, &d.partials, (size_t)maxg * kMaxPartials));
   TRY(dalloc(p, &d.partials2, (size_t)maxg * kMaxPartials));
+  for (int f = 0; f < (p->mixed ? 2 : 1); ++f) {
+    const long long rb = resident_bytes(m, n, nz, f ? 4 : 8);
+    if (rb > 0) TRY(dalloc(p, &p->res[f].block, (size_t)rb));
+  }
   d.A = Csr{d.A_rp, d.A_ci, d.A_v};
   d.At = Csr{d.At_rp, d.At_ci, d.At_v};
   return LP_OK;
@@ -692,6 +710,7 @@ int set_state_impl(lp_problem* p, const double* vn, const double* vm, const doub
   hs.checked0 = scal[13] != 0.0;
   hs.pend_p = hs.pend_d = 0;
   hs.status = 0;
+  hs.fault = 0;
   hs.counter = 0;
   hs.restart_action = 0;
   hs.adopt_avg = 0;
@@ -803,7 +822,7 @@ int create_impl(int32_t m, int32_t n, int64_t nnz, const int64_t* row_ptr, const
     }
     p->own_stream = true;
   }
-  if (cudaMallocHost(&p->h_status, sizeof(int)) != cudaSuccess ||
+  if (cudaMallocHost(&p->h_status, 2 * sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&p->h_scratch, 8 * sizeof(double)) != cudaSuccess) {
     set_err(p, LP_ERR_OOM, "pinned host allocation failed");
     return fail(LP_ERR_OOM);
@@ -917,6 +936,51 @@ int maybe_log(lp_problem* p) {
   return LP_OK;
 }
 
+// The resident plan of the current precision, built at its first use; null
+// when the problem takes the two-kernel path.
+const ResPlan* resident_plan(lp_problem* p, int* rc) {
+  *rc = LP_OK;
+  lp_problem::Resident& R = p->res[p->fp32_phase ? 1 : 0];
+  if (p->opt.kernel_timing || !R.block) return nullptr;  // (timing samples the two step kernels)
+  if (R.tried) return R.ok ? &R.plan : nullptr;
+  R.tried = true;
+  auto build = [&]() -> int {
+    const int esize = p->fp32_phase ? 4 : 8;
+    int limit = 0;
+    CK(resident_smem_limit(p->device, &limit));
+    std::vector<int> head[2];
+    for (int which = 0; which < 2; ++which) {
+      head[which].assign((size_t)resident_long_rows(which ? p->d.binsAt : p->d.binsA) + 1, 0);
+      CK(cudaMemcpyAsync(head[which].data(), which ? p->d.At_rp : p->d.A_rp, sizeof(int) * head[which].size(),
+                         cudaMemcpyDeviceToHost, p->stream));
+    }
+    CK(cudaStreamSynchronize(p->stream));
+    ResHost h;
+    if (!resident_build(p->d.binsA, p->d.binsAt, p->d.m, p->d.n, p->nnz, head[0], head[1], esize, p->sms, limit, h))
+      return LP_OK;
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t ib = h.items.size() * sizeof(ResItem), cb = h.cta.size() * sizeof(ResCta);
+    const size_t o1 = up(ib), o2 = o1 + up(cb), o3 = o2 + up(16 * (8 * (size_t)h.plan.G + 8));
+    const size_t o4 = o3 + up((size_t)(p->d.n + 2LL * p->d.m) * 2 * esize);
+    if ((long long)(o4 + 256) > resident_bytes(p->d.m, p->d.n, p->nnz, esize)) return LP_OK;
+    CK(cudaMemcpyAsync(R.block, h.items.data(), ib, cudaMemcpyHostToDevice, p->stream));
+    CK(cudaMemcpyAsync(R.block + o1, h.cta.data(), cb, cudaMemcpyHostToDevice, p->stream));
+    CK(cudaMemsetAsync(R.block + o2, 0, o4 + 256 - o2, p->stream));
+    CK(cudaStreamSynchronize(p->stream));
+    h.plan.items = reinterpret_cast<const ResItem*>(R.block);
+    h.plan.cta = reinterpret_cast<const ResCta*>(R.block + o1);
+    h.plan.rec = reinterpret_cast<ulonglong2*>(R.block + o2);
+    h.plan.ctl = h.plan.rec + 7 * h.plan.G;
+    h.plan.gx = R.block + o3;
+    h.plan.bar = reinterpret_cast<unsigned int*>(R.block + o4);
+    R.plan = h.plan;
+    R.ok = true;
+    return LP_OK;
+  };
+  *rc = build();
+  return R.ok ? &R.plan : nullptr;
+}
+
 int solve_impl(lp_problem* p, double tol, int64_t iter_limit, int32_t* status_out) {
   TRY(select_device(p));
   const auto t0 = std::chrono::steady_clock::now();
@@ -943,7 +1007,29 @@ int solve_impl(lp_problem* p, double tol, int64_t iter_limit, int32_t* status_ou
     const long long to_boundary = ce - p->host_attempts % ce;
     const long long remaining = iter_limit - p->host_attempts;
     bool checked = false;
-    if (p->opt.use_graph && to_boundary == ce && remaining >= ce) {
+    int rrc = LP_OK;
+    const ResPlan* plan = resident_plan(p, &rrc);
+    TRY(rrc);
+    if (plan) {
+      const long long nrun = to_boundary < remaining ? to_boundary : remaining;
+      checked = nrun == to_boundary;
+      int fault = 0;
+      {
+        SmLease lease(p->device, p->sms, plan->G > 1 ? plan->G : 0, plan->G);
+        CK(launch_resident(p->d, p->prm, *plan, fp32, (int)nrun, p->stream));
+        if (checked) launch_check(p->d, p->prm, 0, fp32, p->stream);
+        CK(cudaGetLastError());
+        TRY(read_status(p, &status, &fault));
+      }
+      if (fault) {
+        CK(cudaMemsetAsync(&p->d.st->fault, 0, sizeof(int), p->stream));
+        p->res[fp32 ? 1 : 0].ok = false;  // the two-kernel path from here on
+        if (fault == 1) return set_err(p, LP_ERR_CUDA, "a resident check period gave up waiting for its CTAs");
+        continue;  // nothing ran
+      }
+      p->launches += 1 + (checked ? check_kernel_count() : 0);
+      p->host_attempts += nrun;
+    } else if (p->opt.use_graph && to_boundary == ce && remaining >= ce) {
       TRY(capture_graph(p, fp32));
       CK(cudaGraphLaunch(fp32 ? p->gexec32 : p->gexec, p->stream));
       p->launches += 2LL * ce + check_kernel_count();
@@ -1208,6 +1294,7 @@ int lp_memory_bytes(int32_t m, int32_t n, int64_t nnz, const lp_options* opt, in
   // padding of the last slices of kSellMaxLen + 1 bins)
   const long long SE = nnz + (kSellMaxLen + 1LL) * 31 * kSellMaxLen;
   t += 2 * (r(4LL * SE) + r(8LL * SE) + (o.precision == LP_PREC_MIXED ? r(4LL * SE) : 0));
+  t += r(resident_bytes(m, n, nnz, 8)) + (o.precision == LP_PREC_MIXED ? r(resident_bytes(m, n, nnz, 4)) : 0);
   *bytes = t;
   return LP_OK;
 }

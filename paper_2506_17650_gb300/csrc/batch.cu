@@ -29,6 +29,7 @@
 #include "common.cuh"
 #include "host_layout.hpp"
 #include "ops.cuh"
+#include "resident.hpp"
 #include "spmv.cuh"
 
 namespace cg = cooperative_groups;
@@ -530,10 +531,24 @@ int build_schedule(lp_batch* b, const std::vector<int>& active, int total_ctas, 
   return LP_OK;
 }
 
+// CTAs of the batched kernel that fit on the GPU at once, in clusters of b->cluster.
+int resident_ctas(lp_batch* b, cudaLaunchConfig_t& cfg, int* total) {
+  const int C = b->cluster;
+  int max_clusters = 0;
+  cfg.gridDim = dim3(C, 1, 1);
+  cudaError_t e = cudaOccupancyMaxActiveClusters(&max_clusters, batch_round_kernel, &cfg);
+  if (e != cudaSuccess || max_clusters < 1)
+    return berr(b, LP_ERR_CUDA, std::string("cluster size ") + std::to_string(C) + " cannot be launched: " +
+                                    cudaGetErrorString(e));
+  *total = max_clusters * C;
+  return LP_OK;
+}
+
 int launch_round(lp_batch* b, const std::vector<int>& active, int attempts) {
   if (active.empty()) return LP_OK;
   const int C = b->cluster;
-  // CTAs: as many clusters as fit at once (persistent)
+  // CTAs: as many clusters as fit at once (persistent) on the SMs that no
+  // resident solve holds; which CTA runs a member does not change its result
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -545,15 +560,15 @@ int launch_round(lp_batch* b, const std::vector<int>& active, int attempts) {
   cfg.stream = b->stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  int max_clusters = 0;
-  cfg.gridDim = dim3(C, 1, 1);
-  cudaError_t e = cudaOccupancyMaxActiveClusters(&max_clusters, batch_round_kernel, &cfg);
-  if (e != cudaSuccess || max_clusters < 1)
-    return berr(b, LP_ERR_CUDA, std::string("cluster size ") + std::to_string(C) + " cannot be launched: " +
-                                    cudaGetErrorString(e));
-  const int total = max_clusters * C;
+  int most = 0;
+  int rc = resident_ctas(b, cfg, &most);
+  if (rc != LP_OK) return rc;
+  const int per_sm = std::max(1, (most + b->sms - 1) / b->sms);
+  const int least = (std::min(most, 2 * C) + per_sm - 1) / per_sm;  // a cluster of each kind
+  SmLease lease(b->device, b->sms, least, std::max(least, (most + per_sm - 1) / per_sm));
+  const int total = std::max(1, std::min(most, lease.count * per_sm) / C) * C;
   std::vector<int> h;
-  int rc = build_schedule(b, active, total, h);
+  rc = build_schedule(b, active, total, h);
   if (rc != LP_OK) return rc;
   if (h.size() > b->sched_cap) {
     if (b->d_sched) cudaFree(b->d_sched);
@@ -570,6 +585,7 @@ int launch_round(lp_batch* b, const std::vector<int>& active, int attempts) {
   cfg.gridDim = dim3(total, 1, 1);
   BCK(cudaLaunchKernelEx(&cfg, batch_round_kernel, (const Member*)b->d_members, queue, q0, q1, cw, C, attempts));
   b->launches += 1;
+  BCK(cudaStreamSynchronize(b->stream));  // the SMs are held until the round is over
   return LP_OK;
 }
 

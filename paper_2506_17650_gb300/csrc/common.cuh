@@ -67,6 +67,8 @@ struct Params {
 struct DevState {
   int cur;        // which half of the double buffers holds the current iterate
   int status;     // 0 running, 1 optimal, 4 numerical error
+  int fault;      // resident launches: 1 a barrier gave up, 2 not started (the checks then do nothing)
+  int unused;
   long long k;    // accepted steps
   int k_mod;      // k mod phi (kept with k: no 64-bit division in the step control)
   long long attempts;

@@ -34,6 +34,7 @@ __global__ void __launch_bounds__(kBlock, kCheckBlocksPerSm<V>) check_primal_ker
   constexpr int NV = AVG ? 2 : 1;
   const Vecs<V>& v = vecs<V>(d);
   const DevState* st = d.st;
+  if (st->fault) return;  // the attempts before this check did not all run
   const int cur = st->cur;
   CheckPrimalOp<NV, V> op;
   op.c = v.c; op.l = v.l; op.u = v.u; op.inv_dc = d.inv_dc;
@@ -62,6 +63,7 @@ template <bool AVG, class V>
 __global__ void __launch_bounds__(kBlock, kCheckBlocksPerSm<V>) check_dual_kernel(Dev d, Params prm, int eval_only) {
   __shared__ double smem[kBlock * 8];
   pdl_wait();
+  if (d.st->fault) return;
   __shared__ double fold[kFold * 10];
   const int nfold = fold_begin<10>(d.partials, partial_rows_at<V>(d), fold);
   const Vecs<V>& v = vecs<V>(d);
@@ -130,6 +132,7 @@ __global__ void check_apply_kernel(Dev d) {
   pdl_wait();
   pdl_trigger();
   const DevState s = *d.st;
+  if (s.fault) return;
   apply_decision<V>(d, s, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 

@@ -1,0 +1,134 @@
+// Plan of a resident check period (resident.hpp): how the rows of a problem are
+// split over the CTAs and laid out in their shared memory, and the SMs that
+// co-resident launches hold.  Pure C++ (no CUDA calls), so that it runs and is
+// tested without a GPU.
+#pragma once
+
+#include <condition_variable>
+#include <mutex>
+#include <vector>
+
+#include "layout_types.h"
+
+struct ulonglong2;  // (CUDA vector type)
+
+namespace lpop {
+
+constexpr int kResThreads = 512;
+constexpr int kResWarps = kResThreads / 32;
+constexpr int kResMaxCtas = 160;   // records and tables are sized for this many
+constexpr int kResWide = 16;       // rows of a CTA that all its warps sum together, at most
+constexpr int kResMaxRow = 8192;   // longest row (entries) of a resident problem
+
+// A warp's work: `nrows` consecutive rows from row0 (bin order), local rows
+// from `vec`, entries from `ent` in the CTA's entry arrays.  kind 0: a slice
+// of 32 rows of at most kSellMaxLen entries, one lane each (entry k of its row
+// t at ent + 32 k + t, `len` the longest row; neighbours in bin order have
+// similar lengths, so few lanes idle, and a small matrix needs one slice where
+// slices of one exact length would take many).  kind 2..32: CSR rows of kind
+// lanes each; kind kResThreads: one CSR row summed by the whole CTA.  For
+// those, `len` is the row's index among the CTA's long rows, which are its
+// first local rows.
+struct ResItem {
+  int row0, nrows, len, kind;
+  int ent, vec;
+};
+
+// A CTA's items [p0, p1) of A^T and [d0, d1) of A, long rows (nlp, nld) and rows.
+struct ResCta {
+  int p0, p1, d0, d1;
+  int nlp, nld, rp, rd;
+};
+
+// What the kernel gets (device pointers; sizes are the largest over the CTAs).
+struct ResPlan {
+  const ResItem* items;
+  const ResCta* cta;
+  ulonglong2* rec;    // [7 * G] records of an attempt, field by field
+  ulonglong2* ctl;    // [8 * (G / 8 + 1)] result of the step control, a line for each eight CTAs
+  void* gx;           // words of x+ [n], then of y+ [2][m]
+  unsigned int* bar;  // arrivals, number of the last attempt, start decision, arrivals before this launch
+  int G;
+  int ep, ed, rp, rd, lp, ld, it;  // entries, rows, long rows of A^T / A; items of both
+  int longest;                     // entries of the longest row of A or A^T
+  int smem;                        // dynamic shared memory, bytes
+};
+
+// Byte offsets of a CTA's arrays in dynamic shared memory.
+struct ResLayout {
+  int vp, vd;    // values of A^T / A entries
+  int xp, xd;    // ten vectors per A^T row, eight per A row
+  int wide;      // warps' sums of the CTA-wide rows
+  int red;       // block sums: four fields of kResThreads doubles
+  int cp, cd;    // column indices
+  int lrp;       // first entry of the long rows (A^T rows, then A rows)
+  int gp, gd;    // global rows
+  int it, sense;
+  int lenp, lend;  // lengths of the slices' rows
+  int total;
+};
+
+LPOP_HD inline int up16(int b) { return (b + 15) & ~15; }
+
+LPOP_HD inline ResLayout res_layout(const ResPlan& p, int esize) {
+  ResLayout L;
+  int o = 0;
+  L.vp = o; o += up16(p.ep * esize);
+  L.vd = o; o += up16(p.ed * esize);
+  L.xp = o; o += up16(10 * p.rp * esize);
+  L.xd = o; o += up16(8 * p.rd * esize);
+  L.wide = o; o += kResWide * kResWarps * 8;
+  L.red = o; o += 4 * kResThreads * 8;
+  L.cp = o; o += up16(p.ep * 4);
+  L.cd = o; o += up16(p.ed * 4);
+  L.lrp = o; o += up16((p.lp + p.ld + 2) * 4);
+  L.gp = o; o += up16(p.rp * 4);
+  L.gd = o; o += up16(p.rd * 4);
+  L.it = o; o += up16(p.it * (int)sizeof(ResItem));
+  L.sense = o; o += up16(p.rd);
+  L.lenp = o; o += up16(p.rp);
+  L.lend = o; o += up16(p.rd);
+  L.total = o;
+  return L;
+}
+
+// Whether a problem of this size may be resident with values of `esize`
+// bytes, and the device bytes its plan takes at most.
+bool resident_possible(long long m, long long n, long long nnz, int esize);
+long long resident_bytes(long long m, long long n, long long nnz, int esize);
+
+struct ResHost {
+  std::vector<ResItem> items;
+  std::vector<ResCta> cta;
+  ResPlan plan{};  // without its device pointers
+};
+
+// The plan of a problem's rows (bin tables of A and A^T) for values of
+// `esize` bytes, at most `sms` CTAs and `smem_limit` bytes each.  head_a /
+// head_at: row pointers of the rows before the first sliced row.  Returns
+// false when the problem does not fit.
+bool resident_build(const BinTable& binsA, const BinTable& binsAt, long long m, long long n, long long nnz,
+                    const std::vector<int>& head_a, const std::vector<int>& head_at, int esize, int sms,
+                    int smem_limit, ResHost& out);
+int resident_long_rows(const BinTable& bt);  // rows before the first sliced row
+
+// SMs of a device that co-resident kernels hold.  The CTAs of a resident
+// launch wait for one another, so two launches that each got part of the GPU
+// would wait for ever: lp_solve takes the SMs of its launch first, in arrival
+// order, and gives them back when the period has finished; the batched kernel
+// (which would otherwise hold every SM for a whole round) takes what is free.
+class SmTokens {
+ public:
+  explicit SmTokens(int sms) : free_(sms) {}
+  // Takes between `least` and `most` SMs, waiting for `least` and for earlier callers.
+  int acquire(int least, int most);
+  void release(int count);
+
+ private:
+  std::mutex mu_;
+  std::condition_variable cv_;
+  int free_;
+  unsigned long long next_ = 0, serving_ = 0;
+};
+
+}  // namespace lpop
