@@ -11,6 +11,8 @@
 // are assigned to teams longest-first by nonzero count.  The team's CTAs hold
 // the member's solver state in shared memory and run the same single-thread
 // control code, so their decisions agree exactly.
+// Blocks of kGroups groups of kBlock threads, each walking its own work units.
+#define LPOP_ROW_GROUPS
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -54,34 +56,41 @@ struct Member {
   Params prm;
 };
 
+// Groups of kBlock threads per CTA.  A member's attempt on one CTA is bound by
+// the latency of its loads and gathers, and one group (8 warps on an SM) left
+// most of them exposed.  256 LPs (2k..300k nonzeros) in one call, mixed, 128
+// attempts: 139.8 ms with one group, 86.8 with two, 75.8 with three, 76.1 with
+// four (64 registers); 64 LPs in clusters of 4, FP64: 34.7, 25.0, 21.9, 22.4 ms.
+constexpr int kGroups = 3;
 constexpr int kSlots = 32;  // team partial slots: primal 3 | dual 4 | check 10 + 8
 
+// This thread among its CTA's, and whether it is the one that runs the control code.
+__device__ __forceinline__ int cta_thread() { return (int)(threadIdx.y * kBlock + threadIdx.x); }
+__device__ __forceinline__ bool cta_first() { return threadIdx.x == 0 && threadIdx.y == 0; }
+
+// Team-wide sums of v (valid in the CTA's first thread): each group's in its
+// slots, then all groups of all CTAs in rank order.  blk: 4 kBlock doubles per group.
 template <int N>
-__device__ void team_reduce(double (&v)[N], double* blk, double* slot, int T, bool wide) {
+__device__ void team_reduce(double (&v)[N], double* blk, double (*slots)[kSlots], int first, int T, bool wide) {
   if (N <= 4) block_sum_smem<N>(v, blk);
   else block_sum<N>(v, blk);
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int q = 0; q < N; ++q) slot[q] = v[q];
+    for (int q = 0; q < N; ++q) slots[threadIdx.y][first + q] = v[q];
   }
   if (wide) cg::this_cluster().sync();
   else __syncthreads();
-  double tot[N];
+  if (!cta_first()) return;
 #pragma unroll
-  for (int q = 0; q < N; ++q) tot[q] = 0.0;
-  if (wide) {
-    cg::cluster_group cl = cg::this_cluster();
-    for (int r = 0; r < T; ++r) {
-      const double* rs = cl.map_shared_rank(slot, r);
+  for (int q = 0; q < N; ++q) v[q] = 0.0;
+  for (int r = 0; r < T; ++r) {
+    double(*rs)[kSlots] = wide ? cg::this_cluster().map_shared_rank(slots, r) : slots;
 #pragma unroll
-      for (int q = 0; q < N; ++q) tot[q] += rs[q];
+    for (int k = 0; k < kGroups; ++k) {
+#pragma unroll
+      for (int q = 0; q < N; ++q) v[q] += rs[k][first + q];
     }
-  } else {
-#pragma unroll
-    for (int q = 0; q < N; ++q) tot[q] = slot[q];
   }
-#pragma unroll
-  for (int q = 0; q < N; ++q) v[q] = tot[q];
 }
 
 __device__ __forceinline__ void team_sync(bool wide) {
@@ -100,7 +109,7 @@ struct StoreRowOp {
 // next to the attempts, whose loop should stay in the instruction caches.
 template <class V>
 __device__ __noinline__ void team_check(const Dev& d, const Params& prm, DevState& s, int rank, int T, bool wide, double* blk,
-                           double* slots, int eval_only = 0) {
+                           double (*slots)[kSlots], int eval_only = 0) {
   const Vecs<V>& v = vecs<V>(d);
   const int cur = s.cur;
   const bool avg = prm.mode == kPdlp && s.wsum > 0.0;
@@ -118,7 +127,7 @@ __device__ __noinline__ void team_check(const Dev& d, const Params& prm, DevStat
     g.x[1] = v.ybar[cur];
     g.n = d.m;
     g.bad = d.bad_gathers;
-    for_each_row_range<2, V, double>(d.binsAt, csr_at<V>(d), g, op, blk, rank, T);
+    for_each_row_range<2, V, double>(d.binsAt, csr_at<V>(d), g, op, blk, rank * kGroups + (int)threadIdx.y, T * kGroups);
 #pragma unroll
     for (int q = 0; q < 10; ++q) p1[q] = op.acc[q];
   } else {
@@ -133,11 +142,11 @@ __device__ __noinline__ void team_check(const Dev& d, const Params& prm, DevStat
     g.x[0] = v.y[cur];
     g.n = d.m;
     g.bad = d.bad_gathers;
-    for_each_row_range<1, V, double>(d.binsAt, csr_at<V>(d), g, op, blk, rank, T);
+    for_each_row_range<1, V, double>(d.binsAt, csr_at<V>(d), g, op, blk, rank * kGroups + (int)threadIdx.y, T * kGroups);
 #pragma unroll
     for (int q = 0; q < 10; ++q) p1[q] = op.acc[q];
   }
-  team_reduce<10>(p1, blk, slots + 7, T, wide);
+  team_reduce<10>(p1, blk, slots, 7, T, wide);
   {
     CheckDualOp<V> op;
     op.b = v.b; op.inv_dr = d.inv_dr; op.sense = d.sense;
@@ -152,21 +161,21 @@ __device__ __noinline__ void team_check(const Dev& d, const Params& prm, DevStat
       g.x[0] = v.xbar[cur];
       g.n = d.n;
       g.bad = d.bad_gathers;
-      for_each_row_range<1, V, double>(d.binsA, csr_a<V>(d), g, op, blk, rank, T);
+      for_each_row_range<1, V, double>(d.binsA, csr_a<V>(d), g, op, blk, rank * kGroups + (int)threadIdx.y, T * kGroups);
     } else {
       const double s0[1] = {0.0};
-      for (int i = rank * blockDim.x + threadIdx.x; i < d.m; i += T * blockDim.x) op.row(i, s0);
+      for (int i = rank * kGroups * kBlock + cta_thread(); i < d.m; i += T * kGroups * kBlock) op.row(i, s0);
     }
 #pragma unroll
     for (int q = 0; q < 8; ++q) p2[q] = op.acc[q];
   }
-  team_reduce<8>(p2, blk, slots + 17, T, wide);
-  if (threadIdx.x == 0) {
+  team_reduce<8>(p2, blk, slots, 17, T, wide);
+  if (cta_first()) {
     check_control(&s, prm, p1, p2, eval_only, avg ? 1 : 0);
     refresh_derived(s, prm.phi, prm.sched);
   }
   __syncthreads();
-  apply_decision<V>(d, s, rank * blockDim.x + threadIdx.x, T * blockDim.x);
+  apply_decision<V>(d, s, rank * kGroups * kBlock + cta_thread(), T * kGroups * kBlock);
   team_sync(wide);
 }
 
@@ -175,7 +184,7 @@ __device__ __noinline__ void team_promote(const Dev& d, const DevState& s, int r
   const Vecs<float>& a = d.f32;
   const Vecs<double>& b = d.f64;
   const int cur = s.cur;
-  const int start = rank * blockDim.x + threadIdx.x, stride = T * blockDim.x;
+  const int start = rank * kGroups * kBlock + cta_thread(), stride = T * kGroups * kBlock;
   for (int j = start; j < d.n; j += stride) {
     b.x[cur][j] = a.x[cur][j];
     b.xbar[cur][j] = a.xbar[cur][j];
@@ -201,15 +210,15 @@ __device__ __noinline__ void team_promote(const Dev& d, const DevState& s, int r
   g.x[0] = b.x[cur];
   g.n = d.n;
   g.bad = d.bad_gathers;
-  for_each_row_range<1, double, double>(d.binsA, d.A, g, op, blk, rank, T);
+  for_each_row_range<1, double, double>(d.binsA, d.A, g, op, blk, rank * kGroups + (int)threadIdx.y, T * kGroups);
   team_sync(wide);
 }
 
 // The FP32 phase reached the tolerance against the FP32 copy of A~: end the
 // phase and let an FP64 termination test of the promoted point decide.
 __device__ __noinline__ void team_certify(const Dev& d, const Params& prm, DevState& s, int rank, int T, bool wide, double* blk,
-                             double* slots) {
-  if (threadIdx.x == 0) {
+                             double (*slots)[kSlots]) {
+  if (cta_first()) {
     s.status = 0;
     s.phase32 = 0;
   }
@@ -222,7 +231,7 @@ __device__ __noinline__ void team_certify(const Dev& d, const Params& prm, DevSt
 // the member handed over from FP32 to FP64 with attempts left.
 template <class V>
 __device__ bool team_round(const Member& mb, DevState& s, int& budget, int rank, int T, bool wide, double* blk,
-                           double* slots) {
+                           double (*slots)[kSlots]) {
   const Dev& d = mb.d;
   const Params& prm = mb.prm;
   const Vecs<V>& v = vecs<V>(d);
@@ -250,10 +259,10 @@ __device__ bool team_round(const Member& mb, DevState& s, int& budget, int rank,
       g.x[0] = v.y[cur];
       g.n = d.m;
       g.bad = d.bad_gathers;
-      for_each_row_range<1, V, V>(d.binsAt, csr_at<V>(d), g, op, blk, rank, T);
+      for_each_row_range<1, V, V>(d.binsAt, csr_at<V>(d), g, op, blk, rank * kGroups + (int)threadIdx.y, T * kGroups);
       t1[0] = op.acc[0]; t1[1] = op.acc[1]; t1[2] = op.acc[2];
     }
-    team_reduce<3>(t1, blk, slots + 0, T, wide);
+    team_reduce<3>(t1, blk, slots, 0, T, wide);
     {
       DualOp<V> op;
       op.sc = read_scalars<V>(&s, false);
@@ -268,11 +277,11 @@ __device__ bool team_round(const Member& mb, DevState& s, int& budget, int rank,
       g.x[0] = v.x[nxt];
       g.n = d.n;
       g.bad = d.bad_gathers;
-      for_each_row_range<1, V, V>(d.binsA, csr_a<V>(d), g, op, blk, rank, T);
+      for_each_row_range<1, V, V>(d.binsA, csr_a<V>(d), g, op, blk, rank * kGroups + (int)threadIdx.y, T * kGroups);
       t2[0] = op.acc[0]; t2[1] = op.acc[1]; t2[2] = op.acc[2]; t2[3] = op.acc[3];
     }
-    team_reduce<4>(t2, blk, slots + 3, T, wide);
-    if (threadIdx.x == 0) {
+    team_reduce<4>(t2, blk, slots, 3, T, wide);
+    if (cta_first()) {
       double f1, f2;
       step_factors(d.step_tab, s.attempts + 1, &f1, &f2);
       step_control_state(s, prm, f1, f2, t1, t2);
@@ -288,7 +297,7 @@ __device__ bool team_round(const Member& mb, DevState& s, int& budget, int rank,
       if (s.status != 0) break;
       if (sizeof(V) == sizeof(float) && s.phase32) {
         // mixed precision hand-over: at refine_tol, or after refine_stall checks without a 10% gain
-        if (threadIdx.x == 0) {
+        if (cta_first()) {
           const double kkt = fmax(s.rel_pres, fmax(s.rel_dres, s.rel_gap));
           if (kkt < 0.9 * s.best_kkt) {
             s.best_kkt = kkt;
@@ -309,13 +318,14 @@ __device__ bool team_round(const Member& mb, DevState& s, int& budget, int rank,
   return false;
 }
 
-__global__ void __launch_bounds__(kBlock) batch_round_kernel(const Member* members, const int* queue,
+__global__ void __launch_bounds__(kGroups* kBlock) batch_round_kernel(const Member* members, const int* queue,
                                                              const int* cta_q0, const int* cta_q1,
                                                              const int* cluster_wide, int C, int attempts) {
   __shared__ Member mb;
   __shared__ DevState s;
-  __shared__ double slots[kSlots];
-  __shared__ double blk[kBlock * 4];
+  __shared__ double slots[kGroups][kSlots];
+  __shared__ double group_blk[kGroups][kBlock * 4];
+  double* const blk = group_blk[threadIdx.y];
   const int cid = blockIdx.x / C;
   const int crank = blockIdx.x % C;
   const bool wide = C > 1 && cluster_wide[cid] != 0;
@@ -327,10 +337,10 @@ __global__ void __launch_bounds__(kBlock) batch_round_kernel(const Member* membe
     {
       const int* src = reinterpret_cast<const int*>(members + id);
       int* dst = reinterpret_cast<int*>(&mb);
-      for (int w = threadIdx.x; w < (int)(sizeof(Member) / sizeof(int)); w += blockDim.x) dst[w] = src[w];
+      for (int w = cta_thread(); w < (int)(sizeof(Member) / sizeof(int)); w += kGroups * kBlock) dst[w] = src[w];
     }
     __syncthreads();
-    if (threadIdx.x == 0) s = *mb.d.st;
+    if (cta_first()) s = *mb.d.st;
     __syncthreads();
     int budget = attempts;
     if (s.status == 0) {
@@ -341,7 +351,7 @@ __global__ void __launch_bounds__(kBlock) batch_round_kernel(const Member* membe
         team_round<double>(mb, s, budget, rank, T, wide, blk, slots);
       }
     }
-    if (rank == 0 && threadIdx.x == 0) *mb.d.st = s;
+    if (rank == 0 && cta_first()) *mb.d.st = s;
     team_sync(wide);
   }
 }
@@ -555,7 +565,7 @@ int launch_round(lp_batch* b, const std::vector<int>& active, int attempts) {
   attr[0].val.clusterDim.x = C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  cfg.blockDim = dim3(kBlock, 1, 1);
+  cfg.blockDim = dim3(kBlock, kGroups, 1);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = b->stream;
   cfg.attrs = attr;

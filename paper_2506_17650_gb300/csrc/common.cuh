@@ -221,6 +221,17 @@ __host__ __device__ inline CsrT<V> csr_a(const Dev& d) { return CsrT<V>{d.A_rp, 
 template <class V>
 __host__ __device__ inline CsrT<V> csr_at(const Dev& d) { return CsrT<V>{d.At_rp, d.At_ci, vecs<V>(d).Atv}; }
 
+// Barrier of the kBlock threads that walk work units together: the block, or
+// -- where a kernel's blocks hold several such groups, as rows of a
+// two-dimensional block (LPOP_ROW_GROUPS) -- the group.
+static __device__ __forceinline__ void row_sync() {
+#ifdef LPOP_ROW_GROUPS
+  asm volatile("bar.sync %0, %1;" ::"r"(threadIdx.y + 1), "n"(kBlock) : "memory");
+#else
+  __syncthreads();
+#endif
+}
+
 // ---------------------------------------------------------------------------
 // Block reductions (fixed shuffle tree then fixed smem order: deterministic)
 // ---------------------------------------------------------------------------
@@ -232,12 +243,12 @@ __device__ inline void block_sum(T (&v)[N], T* smem /* [32 * N] */) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
   }
-  __syncthreads();
+  row_sync();
   if (lane == 0) {
 #pragma unroll
     for (int q = 0; q < N; ++q) smem[warp * N + q] = v[q];
   }
-  __syncthreads();
+  row_sync();
   const int nw = blockDim.x >> 5;
   if (warp == 0) {
 #pragma unroll
@@ -248,7 +259,7 @@ __device__ inline void block_sum(T (&v)[N], T* smem /* [32 * N] */) {
       v[q] = t;  // valid in warp 0
     }
   }
-  __syncthreads();
+  row_sync();
 }
 
 // Block sum through shared memory: every thread stores its N values, then one
@@ -260,7 +271,7 @@ __device__ inline void block_sum_smem(double (&v)[N], double* smem) {
   const int tid = threadIdx.x;
 #pragma unroll
   for (int q = 0; q < N; ++q) smem[q * 256 + tid] = v[q];
-  __syncthreads();
+  row_sync();
   if (tid < 32) {
 #pragma unroll
     for (int q = 0; q < N; ++q) {
@@ -274,7 +285,7 @@ __device__ inline void block_sum_smem(double (&v)[N], double* smem) {
       v[q] = t;
     }
   }
-  __syncthreads();
+  row_sync();
 }
 
 // Order-preserving integer key of a double (not NaN): comparisons of keys
