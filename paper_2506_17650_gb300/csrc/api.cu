@@ -419,6 +419,16 @@ int sliced_unit_rows(const BinTable& bt, int cap, int sms) {
   return best;
 }
 
+// The A-row step kernel holds the x of the longest columns (which come first)
+// in shared memory when they have at least a quarter of the entries and every
+// SM has its full blocks.  Entries per block: on the 30M-nonzero power-law LP
+// (about half of all entries are in its 1,024 longest columns) the FP64 kernel
+// took 163.2 us without, 151.6 with 256 to 1,536 and 166.8 with 2,048, the FP32
+// one 129.8 without, 123.5 with 2,048 or 3,072, 113.9 with 4,096 and 117.1 with
+// 5,120.
+constexpr int kHotX = 1024;
+constexpr int kHotX32 = 4096;
+
 // Device buffers and the layout: the CSR copies of A and A^T and the vectors
 // in bin order are built on the device from the caller's (valid, canonical)
 // arrays, with scratch taken from the arena and given back afterwards.
@@ -520,6 +530,19 @@ int upload(lp_problem* p, int m, int n, long long nz, const int64_t* row_ptr, co
     CK(cudaMemcpyAsync(su, units.data(), sizeof(int) * units.size(), cudaMemcpyHostToDevice, p->stream));
     CK(cudaMemsetAsync(bt.ticket, 0, sizeof(unsigned int) * bt.seg_rows, p->stream));
     bt.seg_unit = su;
+  }
+  // x of the longest columns, for the A-row step kernel's gathers
+  {
+    const int hot = kHotX, hot32 = kHotX32;
+    d.hot = d.hot32 = 0;
+    if (n > hot32 && d.gridA >= cap_d) {
+      int entries[2] = {0, 0};
+      for (int k = 0; k < 2; ++k)
+        CK(cudaMemcpyAsync(entries + k, d.At_rp + (k ? hot32 : hot), sizeof(int), cudaMemcpyDeviceToHost, p->stream));
+      CK(cudaStreamSynchronize(p->stream));
+      if (4LL * entries[0] >= nz) d.hot = hot;
+      if (4LL * entries[1] >= nz) d.hot32 = hot32;
+    }
   }
   for (int which = 0; which < 2; ++which) {  // Ruiz units: whole-block rows in chunks, then warp and thread rows
     const std::vector<int>& head = which ? lay.At_head : lay.A_head;

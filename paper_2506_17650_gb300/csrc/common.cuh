@@ -184,6 +184,7 @@ struct Dev {
   unsigned int* bad_gathers;  // checked builds: gathers whose index fell outside the vector
   BinTable binsA, binsAt;
   int gridA, gridAt;      // blocks launched for the A / A^T row kernels (FP64)
+  int hot, hot32;         // first entries of x that a block of the A-row step kernel holds in shared memory (FP64, FP32)
   int gridA32, gridAt32;  // the same for the FP32 kernels (fewer registers, more resident blocks)
   int max_grid;
 };
@@ -452,8 +453,9 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <class... KArgs, class... Args>
-inline void launch_pdl(void (*kernel)(KArgs...), int grid, cudaStream_t s, Args... args) {
+inline void launch_pdl_smem(void (*kernel)(KArgs...), int grid, int smem, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
+  cfg.dynamicSmemBytes = (size_t)smem;
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3(kBlock, 1, 1);
   cfg.stream = s;
@@ -463,6 +465,11 @@ inline void launch_pdl(void (*kernel)(KArgs...), int grid, cudaStream_t s, Args.
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, args...);  // errors surface through cudaGetLastError
+}
+
+template <class... KArgs, class... Args>
+inline void launch_pdl(void (*kernel)(KArgs...), int grid, cudaStream_t s, Args... args) {
+  launch_pdl_smem(kernel, grid, 0, s, args...);
 }
 
 // ---------------------------------------------------------------------------

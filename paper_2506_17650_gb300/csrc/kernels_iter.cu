@@ -22,6 +22,8 @@
 // 1/Sigma are kept as vectors and rewritten only when T / Sigma change),
 // clamps and sign projections on the integer pipes (ordered keys), step
 // scalars precomputed by the control thread, and block sums done by one warp.
+#include <type_traits>
+
 #include "common.cuh"
 #include "ops.cuh"
 #include "spmv.cuh"
@@ -64,8 +66,9 @@ __global__ void __launch_bounds__(kBlock, kStepBlocksPerSm<V>) primal_step_kerne
   pdl_trigger();
 }
 
-template <class V>
+template <class V, bool kHot>
 __global__ void __launch_bounds__(kBlock, kStepBlocksPerSm<V>) dual_step_kernel(Dev d, Params prm) {
+  extern __shared__ __align__(16) unsigned char s_hot[];
   __shared__ double smem[kBlock * 7];
   __shared__ double fold[kFold * 3];
   __shared__ DevState s_st;  // the state does not change until the step control, at the very end
@@ -90,10 +93,19 @@ __global__ void __launch_bounds__(kBlock, kStepBlocksPerSm<V>) dual_step_kernel(
   op.S = v.S; op.invS = v.invS; op.GS = v.GS; op.p = v.p;
   op.yn = v.y[nxt]; op.axn = v.ax[nxt]; op.ybarn = v.ybar[nxt];
   op.acc[0] = op.acc[1] = op.acc[2] = op.acc[3] = V(0);
-  Gather<1, V> g;
+  std::conditional_t<kHot, HotGather<V>, Gather<1, V>> g;
   g.x[0] = v.x[nxt];  // x+ written by the primal kernel
   g.n = d.n;
   g.bad = d.bad_gathers;
+  if constexpr (kHot) {
+    V* const hot = reinterpret_cast<V*>(s_hot);
+    const int nhot = sizeof(V) == 4 ? d.hot32 : d.hot;
+    for (int i = threadIdx.x; i < nhot * (int)sizeof(V) / 16; i += kBlock)
+      reinterpret_cast<int4*>(hot)[i] = __ldg(reinterpret_cast<const int4*>(v.x[nxt]) + i);
+    __syncthreads();
+    g.hot = hot;
+    g.nhot = nhot;
+  }
   for_each_row<1, V, V>(d.binsA, csr_a<V>(d), g, op, smem, row_slots_a<V>(d, d.partials2));
   double a[4] = {(double)op.acc[0], (double)op.acc[1], (double)op.acc[2], (double)op.acc[3]};
   block_sum_smem<4>(a, smem);
@@ -188,8 +200,13 @@ void launch_primal(const Dev& d, const Params& prm, bool fp32, cudaStream_t s) {
 }
 
 void launch_dual(const Dev& d, const Params& prm, bool fp32, cudaStream_t s) {
-  if (fp32) launch_pdl(dual_step_kernel<float>, d.gridA32, s, d, prm);
-  else launch_pdl(dual_step_kernel<double>, d.gridA, s, d, prm);
+  if (fp32) {
+    if (d.hot32 > 0) launch_pdl_smem(dual_step_kernel<float, true>, d.gridA32, d.hot32 * (int)sizeof(float), s, d, prm);
+    else launch_pdl(dual_step_kernel<float, false>, d.gridA32, s, d, prm);
+  } else {
+    if (d.hot > 0) launch_pdl_smem(dual_step_kernel<double, true>, d.gridA, d.hot * (int)sizeof(double), s, d, prm);
+    else launch_pdl(dual_step_kernel<double, false>, d.gridA, s, d, prm);
+  }
 }
 
 void launch_flush_update(const Dev& d, const Params& prm, bool fp32, cudaStream_t s) {
@@ -212,9 +229,9 @@ void row_kernel_blocks_per_sm(int* primal, int* dual, int* primal32, int* dual32
     return a;
   };
   *primal = occ(primal_step_kernel<double>);
-  *dual = occ(dual_step_kernel<double>);
+  *dual = occ(dual_step_kernel<double, false>);
   *primal32 = occ(primal_step_kernel<float>);
-  *dual32 = occ(dual_step_kernel<float>);
+  *dual32 = occ(dual_step_kernel<float, false>);
 }
 
 }  // namespace lpop

@@ -45,6 +45,22 @@ __device__ __forceinline__ V gather(const Gather<NV, V>& g, int q, int c) {
   return __ldg(g.x[q] + c);
 }
 
+// A gather whose first nhot entries are in shared memory.  Columns are stored
+// longest first, so with power-law degrees the first few thousand entries of x
+// are about half of all that the rows of A gather; from shared memory a warp's
+// gather takes its bank conflicts (about 7 cycles in FP64) instead of a cycle
+// of the load unit for each lane's line.
+template <class V>
+struct HotGather : Gather<1, V> {
+  const V* hot;
+  int nhot;
+};
+
+template <class V>
+__device__ __forceinline__ V gather(const HotGather<V>& g, int q, int c) {
+  return (unsigned)c < (unsigned)g.nhot ? g.hot[c] : gather(static_cast<const Gather<1, V>&>(g), q, c);
+}
+
 // Ops that keep per-block reduction accumulators (member `acc`).
 template <class Op, class = void>
 struct HasAcc : std::false_type {};
@@ -70,8 +86,8 @@ struct ReadsCsrOnly<Op, std::void_t<decltype(Op::kCsrOnly)>> : std::true_type {}
 constexpr int kChunk = 8;
 
 // s[q] += sum over this lane's entries k = k0 + u * stride (u < kChunk, k < end), in order of k.
-template <int NV, class V, class Acc>
-__device__ __forceinline__ void chunk_dot(int k0, int end, int stride, const CsrT<V>& M, const Gather<NV, V>& g,
+template <int NV, class V, class Acc, class G>
+__device__ __forceinline__ void chunk_dot(int k0, int end, int stride, const CsrT<V>& M, const G& g,
                                           Acc (&s)[NV]) {
   int c[kChunk];
   Acc a[kChunk];
@@ -101,8 +117,8 @@ __device__ __forceinline__ void chunk_dot(int k0, int end, int stride, const Csr
 }
 
 // Rows first + tid / W < row_end, W lanes each.
-template <int W, int NV, class V, class Acc, class Op>
-__device__ __forceinline__ void vec_rows(int first, int row_end, const CsrT<V>& M, const Gather<NV, V>& g,
+template <int W, int NV, class V, class Acc, class G, class Op>
+__device__ __forceinline__ void vec_rows(int first, int row_end, const CsrT<V>& M, const G& g,
                                          Op& op) {
   const int row = first + (int)threadIdx.x / W;
   const int lane = (int)threadIdx.x % W;
@@ -136,8 +152,8 @@ __device__ __forceinline__ const float* sell_values<float>(const BinTable& bt) {
 // the sliced copy.  Called by consecutive threads for consecutive rows, so the
 // loop bound is the same for the whole warp and the loads of a warp are
 // contiguous; the entries are added in row order, as in the CSR path.
-template <int NV, class V, class Acc, class Op>
-__device__ __forceinline__ void sell_rows_at(const BinTable& bt, const Bin& B, int i, const Gather<NV, V>& g,
+template <int NV, class V, class Acc, class G, class Op>
+__device__ __forceinline__ void sell_rows_at(const BinTable& bt, const Bin& B, int i, const G& g,
                                              Op& op) {
   const int row = B.row_begin + i;
   if (row >= B.row_end) return;
@@ -174,8 +190,8 @@ __device__ __forceinline__ void sell_rows_at(const BinTable& bt, const Bin& B, i
 
 // A unit of a kSell bin: thread t < R takes row local * R + t of the bin (R
 // rows per unit: kBlock, or fewer when the matrix spreads its rows thinner).
-template <int NV, class V, class Acc, class Op>
-__device__ __forceinline__ void sell_rows(const BinTable& bt, const Bin& B, int local, const Gather<NV, V>& g,
+template <int NV, class V, class Acc, class G, class Op>
+__device__ __forceinline__ void sell_rows(const BinTable& bt, const Bin& B, int local, const G& g,
                                           Op& op) {
   const int R = rows_per_unit(B);
   if ((int)threadIdx.x < R) sell_rows_at<NV, V, Acc>(bt, B, local * R + (int)threadIdx.x, g, op);
@@ -187,8 +203,8 @@ __device__ __forceinline__ void sell_rows(const BinTable& bt, const Bin& B, int 
 // arithmetic, so that the two rows' FP64 chains interleave.  The second row's
 // reduction terms are kept apart and added to the thread's accumulators after
 // the pair (a fixed order).
-template <int NV, class V, class Acc, class Op>
-__device__ __forceinline__ void sell_rows_pair(const BinTable& bt, const Bin& B, int local, const Gather<NV, V>& g,
+template <int NV, class V, class Acc, class G, class Op>
+__device__ __forceinline__ void sell_rows_pair(const BinTable& bt, const Bin& B, int local, const G& g,
                                                Op& op) {
   constexpr int C = kPairMaxLen;
   const int H = rows_per_unit(B) / 2;  // rows per half unit: thread t < H takes rows t and H + t
@@ -249,8 +265,8 @@ __device__ __forceinline__ void sell_rows_pair(const BinTable& bt, const Bin& B,
 }
 
 // Block-wide FP64 sums of the entries [beg, end) of one row (valid in warp 0).
-template <int NV, class V, class Acc>
-__device__ __forceinline__ void block_dot(int beg, int end, const CsrT<V>& M, const Gather<NV, V>& g, double (&s)[NV],
+template <int NV, class V, class Acc, class G>
+__device__ __forceinline__ void block_dot(int beg, int end, const CsrT<V>& M, const G& g, double (&s)[NV],
                                           double* smem) {
 #pragma unroll
   for (int q = 0; q < NV; ++q) s[q] = 0.0;
@@ -302,9 +318,9 @@ __device__ __forceinline__ void row_into_slot(Op& op, int row, const Acc (&r)[NV
 // last segment adds the segment sums in segment order and runs the epilogue
 // into the row's slot.  Without, the unit of segment 0 takes the whole row and
 // the others do nothing.
-template <int NV, class V, class Acc, class Op>
+template <int NV, class V, class Acc, class G, class Op>
 __device__ __forceinline__ void wide_unit(const BinTable& bt, int local, int row, int seg, const CsrT<V>& M,
-                                          const Gather<NV, V>& g, Op& op, double* smem, double* row_slots) {
+                                          const G& g, Op& op, double* smem, double* row_slots) {
   static_assert(NV <= 2, "segment sums hold up to two vectors");
   const bool split = seg >= 0 && HasAcc<Op>::value && row_slots != nullptr;
   if (!split && seg > 0) return;
@@ -343,8 +359,8 @@ __device__ __forceinline__ void wide_unit(const BinTable& bt, int local, int row
 // Work units first_unit, first_unit + unit_stride, ... of the table (one block
 // per unit at a time).  smem must hold 32 * NV doubles.  row_slots: see
 // segment_unit.
-template <int NV, class V, class Acc, class Op>
-__device__ __forceinline__ void for_each_row_range(const BinTable& bt, const CsrT<V>& M, const Gather<NV, V>& g,
+template <int NV, class V, class Acc, class G, class Op>
+__device__ __forceinline__ void for_each_row_range(const BinTable& bt, const CsrT<V>& M, const G& g,
                                                    Op& op, double* smem, int first_unit, int unit_stride,
                                                    double* row_slots = nullptr) {
   int b = 0;  // units only increase, so the bin search resumes where it stopped
@@ -389,8 +405,8 @@ __device__ __forceinline__ void for_each_row_range(const BinTable& bt, const Csr
 
 // All work units, spread over the grid's blocks in a grid-stride loop (the
 // longest rows are numbered first, so they start first).
-template <int NV, class V, class Acc, class Op>
-__device__ __forceinline__ void for_each_row(const BinTable& bt, const CsrT<V>& M, const Gather<NV, V>& g, Op& op,
+template <int NV, class V, class Acc, class G, class Op>
+__device__ __forceinline__ void for_each_row(const BinTable& bt, const CsrT<V>& M, const G& g, Op& op,
                                              double* smem, double* row_slots = nullptr) {
   for_each_row_range<NV, V, Acc>(bt, M, g, op, smem, blockIdx.x, gridDim.x, row_slots);
 }
