@@ -28,6 +28,8 @@ using namespace lpop;
 namespace lpop {
 void launch_scatter_perm(double* out, const double* a, const double* f, const int* perm, int n, cudaStream_t s);
 void launch_gather_perm(double* out, const double* a, const int* perm, int n, cudaStream_t s);
+void launch_result(const Dev& d, bool fp32, double* x, double* y, const int* prow, const int* pcol, cudaStream_t s);
+void launch_begin_solve(DevState* st, double tol, cudaStream_t s);
 void row_kernel_blocks_per_sm(int* primal, int* dual, int* primal32, int* dual32);
 }  // namespace lpop
 
@@ -241,8 +243,7 @@ int init_state(lp_problem* p) {
   s0.phase32 = p->mixed ? 1 : 0;
   s0.best_kkt = INFINITY;
   refresh_derived(s0, p->prm.phi, p->prm.sched);
-  CK(cudaMemcpyAsync(p->d.st, &s0, sizeof(s0), cudaMemcpyHostToDevice, p->stream));
-  launch_init_vectors(p->d, p->stream);
+  launch_init_state(p->d, s0, p->stream);
   launch_spmv_binned(p->d.A, p->d.binsA, p->d.gridA, p->d.f64.x[0], p->d.f64.ax[0], p->stream);
   if (p->mixed) launch_demote_state(p->d, p->stream);
   CK(cudaGetLastError());
@@ -1009,10 +1010,8 @@ int solve_impl(lp_problem* p, double tol, int64_t iter_limit, int32_t* status_ou
   const auto t0 = std::chrono::steady_clock::now();
   const int ce = p->opt.check_every;
   // tolerance and a cleared status for this call
-  p->h_scratch[0] = tol;
-  CK(cudaMemcpyAsync(&p->d.st->tol, p->h_scratch, sizeof(double), cudaMemcpyHostToDevice, p->stream));
-  *p->h_status = 0;
-  CK(cudaMemcpyAsync(&p->d.st->status, p->h_status, sizeof(int), cudaMemcpyHostToDevice, p->stream));
+  launch_begin_solve(p->d.st, tol, p->stream);
+  CK(cudaGetLastError());
   int status = 0;
   if (!p->initial_check_done) {
     launch_check(p->d, p->prm, 0, p->fp32_phase, p->stream);
@@ -1201,10 +1200,14 @@ int lp_result(lp_problem* p, double* x, double* y, lp_stats* st) {
   if (!p->solved_once) return set_err(p, LP_ERR_NOT_SOLVED, "lp_result called before lp_solve");
   TRY(select_device(p));
   DevState hs;
+  const int n = p->d.n, m = p->d.m;
+  double* tmp = p->d.work;  // [m + n + 2048]
+  launch_result(p->d, p->fp32_phase, x ? tmp : nullptr, y && m > 0 ? tmp + n : nullptr, p->d_prow, p->d_pcol, p->stream);
+  CK(cudaGetLastError());
   CK(cudaMemcpyAsync(&hs, p->d.st, sizeof(hs), cudaMemcpyDeviceToHost, p->stream));
+  if (x) CK(cudaMemcpyAsync(x, tmp, sizeof(double) * n, cudaMemcpyDeviceToHost, p->stream));
+  if (y && m > 0) CK(cudaMemcpyAsync(y, tmp + n, sizeof(double) * m, cudaMemcpyDeviceToHost, p->stream));
   CK(cudaStreamSynchronize(p->stream));
-  if (x) TRY(download_vec(p, phase_vec(p, p->d.f64.x[hs.cur], p->d.f32.x[hs.cur], p->d.n), p->d.dc, p->d.n, p->d_pcol, x));
-  if (y) TRY(download_vec(p, phase_vec(p, p->d.f64.y[hs.cur], p->d.f32.y[hs.cur], p->d.m), p->d.dr, p->d.m, p->d_prow, y));
   if (st) {
     std::memset(st, 0, sizeof(*st));
     st->pobj = hs.pobj;
@@ -1359,6 +1362,22 @@ __global__ void scatter_perm_kernel(double* out, const double* a, const double* 
     out[perm[i]] = f ? a[i] * f[i] : a[i];
 }
 
+// The tolerance and a cleared status for a solve.
+__global__ void begin_solve_kernel(DevState* st, double tol) {
+  st->tol = tol;
+  st->status = 0;
+}
+
+// The current point in user units and the caller's order (x, y: null to leave out).
+template <class V>
+__global__ void result_kernel(Dev d, double* x, double* y, const int* prow, const int* pcol) {
+  const Vecs<V>& v = vecs<V>(d);
+  const int cur = d.st->cur, t0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  const V *xc = v.x[cur], *yc = v.y[cur];
+  for (int j = t0; x && j < d.n; j += stride) x[pcol[j]] = (double)xc[j] * d.dc[j];
+  for (int i = t0; y && i < d.m; i += stride) y[prow[i]] = (double)yc[i] * d.dr[i];
+}
+
 // out[i] = a[perm[i]]
 __global__ void gather_perm_kernel(double* out, const double* a, const int* perm, int n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) out[i] = a[perm[i]];
@@ -1373,6 +1392,14 @@ int perm_grid(int n) {
 
 void launch_scatter_perm(double* out, const double* a, const double* f, const int* perm, int n, cudaStream_t s) {
   scatter_perm_kernel<<<perm_grid(n), kBlock, 0, s>>>(out, a, f, perm, n);
+}
+
+void launch_begin_solve(DevState* st, double tol, cudaStream_t s) { begin_solve_kernel<<<1, 1, 0, s>>>(st, tol); }
+
+void launch_result(const Dev& d, bool fp32, double* x, double* y, const int* prow, const int* pcol, cudaStream_t s) {
+  const int g = perm_grid(d.n > d.m ? d.n : d.m);
+  if (fp32) result_kernel<float><<<g, kBlock, 0, s>>>(d, x, y, prow, pcol);
+  else result_kernel<double><<<g, kBlock, 0, s>>>(d, x, y, prow, pcol);
 }
 
 void launch_gather_perm(double* out, const double* a, const int* perm, int n, cudaStream_t s) {

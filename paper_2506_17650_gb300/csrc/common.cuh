@@ -526,7 +526,7 @@ void launch_ruiz_apply(const Dev& d, const RuizSplit& a, const RuizSplit& at, do
 void launch_row_powsum(const Csr& M, int rows, int nlong, int split, double beta, int square_root, double* out,
                        cudaStream_t s);
 void launch_scale_problem_vectors(const Dev& d, cudaStream_t s);
-void launch_init_vectors(const Dev& d, cudaStream_t s);
+void launch_init_state(const Dev& d, const DevState& s0, cudaStream_t s);  // vectors and *d.st
 void launch_spmv_binned(const Csr& M, const BinTable& bt, int grid, const double* x, double* y, cudaStream_t s);
 void launch_norm2(const double* v, int n, double* out, cudaStream_t s);  // out[0] = ||v||_2; out[1..1025) scratch
 void launch_absmax(const double* v, long long n, double* out, cudaStream_t s);

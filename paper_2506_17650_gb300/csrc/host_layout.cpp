@@ -14,6 +14,11 @@ namespace lpop {
 namespace {
 
 // Host threads for the layout's parallel phases: every hardware thread, up to 32.
+// Starting one costs about as long as it takes to scan a hundred thousand
+// entries, so a phase gets one per kThreadWork elements of its work: with all
+// of them from 65,536 elements on, the checks of a 60k-nonzero LP spent most of
+// their time starting threads.
+constexpr long long kThreadWork = 1 << 18;
 int layout_threads() {
   const unsigned hw = std::thread::hardware_concurrency();
   return (int)std::min<unsigned>(hw == 0 ? 1u : hw, 32u);
@@ -24,17 +29,17 @@ int layout_threads() {
 // the rows when a range is rows) is large.
 template <class Fn>
 void parallel_ranges(long long count, Fn fn, long long work = -1) {
-  int t = layout_threads();
-  if ((work < 0 ? count : work) < (1 << 16)) t = 1;
+  const int t = (int)std::min<long long>(layout_threads(), (work < 0 ? count : work) / kThreadWork + 1);
   if (t <= 1) {
     fn(0LL, count);
     return;
   }
   std::vector<std::thread> pool;
-  for (int i = 0; i < t; ++i) {
+  for (int i = 1; i < t; ++i) {
     const long long b = count * i / t, e = count * (i + 1) / t;
     pool.emplace_back([=]() { fn(b, e); });
   }
+  fn(0LL, count / t);
   for (auto& th : pool) th.join();
 }
 

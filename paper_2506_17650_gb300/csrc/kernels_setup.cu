@@ -285,8 +285,9 @@ __global__ void __launch_bounds__(kBlock) spmv_kernel(Csr M, BinTable bt, const 
   for_each_row<1, double, double>(bt, M, g, op, smem);
 }
 
-__global__ void init_vectors_kernel(Dev d) {
+__global__ void init_state_kernel(Dev d, DevState s0) {
   const Vecs<double>& v = d.f64;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *d.st = s0;
   const int stride = gridDim.x * blockDim.x;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n; j += stride) {
     const double x0 = fmin(fmax(0.0, v.l[j]), v.u[j]);
@@ -478,8 +479,8 @@ void launch_spmv_binned(const Csr& M, const BinTable& bt, int grid, const double
   if (bt.nunits > 0) spmv_kernel<<<grid, kBlock, 0, s>>>(M, bt, x, y);
 }
 
-void launch_init_vectors(const Dev& d, cudaStream_t s) {
-  init_vectors_kernel<<<grid_for(d.n > d.m ? d.n : d.m), kBlock, 0, s>>>(d);
+void launch_init_state(const Dev& d, const DevState& s0, cudaStream_t s) {
+  init_state_kernel<<<grid_for(d.n > d.m ? d.n : d.m), kBlock, 0, s>>>(d, s0);
 }
 
 }  // namespace lpop
