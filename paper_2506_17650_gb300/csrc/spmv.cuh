@@ -369,7 +369,8 @@ __device__ __forceinline__ void for_each_row_range(const BinTable& bt, const Csr
     const Bin& B = bt.bin[b];
     const int local = u - B.unit_begin;
     const int width = B.width;
-    if (width == kSell && bt.sell_ci) {
+    // (a matrix without entries has sliced rows and no copy, nothing of which is then read)
+    if (width == kSell && (bt.sell_ci || !ReadsCsrOnly<Op>::value)) {
       if (B.len <= kPairMaxLen) {  // units of two halves of H rows (H = kBlock by default)
         if constexpr (AllowsPair<Op>::value) {
           sell_rows_pair<NV, V, Acc>(bt, B, local, g, op);
