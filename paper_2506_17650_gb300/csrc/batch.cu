@@ -248,13 +248,8 @@ __device__ bool team_round(const Member& mb, DevState& s, int& budget, int rank,
     {
       PrimalOp<V> op;
       op.sc = read_scalars<V>(&s, true);
-      const int cur = op.sc.cur, nxt = cur ^ 1;
-      op.prm = prm;
-      op.c = v.c; op.l = v.l; op.u = v.u;
-      op.xc = v.x[cur]; op.xbarc = v.xbar[cur];
-      op.T = v.T; op.invT = v.invT; op.GT = v.GT; op.q = v.q;
-      op.xn = v.x[nxt]; op.xbarn = v.xbar[nxt];
-      op.acc[0] = op.acc[1] = op.acc[2] = V(0);
+      const int cur = op.sc.cur;
+      op.bind(v, prm, cur);
       Gather<1, V> g;
       g.x[0] = v.y[cur];
       g.n = d.m;
@@ -267,12 +262,7 @@ __device__ bool team_round(const Member& mb, DevState& s, int& budget, int rank,
       DualOp<V> op;
       op.sc = read_scalars<V>(&s, false);
       const int cur = op.sc.cur, nxt = cur ^ 1;
-      op.prm = prm;
-      op.b = v.b; op.sense = d.sense;
-      op.axc = v.ax[cur]; op.yc = v.y[cur]; op.ybarc = v.ybar[cur];
-      op.S = v.S; op.invS = v.invS; op.GS = v.GS; op.p = v.p;
-      op.yn = v.y[nxt]; op.axn = v.ax[nxt]; op.ybarn = v.ybar[nxt];
-      op.acc[0] = op.acc[1] = op.acc[2] = op.acc[3] = V(0);
+      op.bind(v, prm, d.sense, cur);
       Gather<1, V> g;
       g.x[0] = v.x[nxt];
       g.n = d.n;

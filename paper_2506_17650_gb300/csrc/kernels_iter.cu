@@ -45,13 +45,8 @@ __global__ void __launch_bounds__(kBlock, kStepBlocksPerSm<V>) primal_step_kerne
   const Vecs<V>& v = vecs<V>(d);
   PrimalOp<V, true> op;
   op.sc = read_scalars<V>(d.st, true);
-  const int cur = op.sc.cur, nxt = cur ^ 1;
-  op.prm = prm;
-  op.c = v.c; op.l = v.l; op.u = v.u;
-  op.xc = v.x[cur]; op.xbarc = v.xbar[cur];
-  op.T = v.T; op.invT = v.invT; op.GT = v.GT; op.q = v.q;
-  op.xn = v.x[nxt]; op.xbarn = v.xbar[nxt];
-  op.acc[0] = op.acc[1] = op.acc[2] = V(0);
+  const int cur = op.sc.cur;
+  op.bind(v, prm, cur);
   Gather<1, V> g;
   g.x[0] = v.y[cur];
   g.n = d.m;
@@ -87,12 +82,7 @@ __global__ void __launch_bounds__(kBlock, kStepBlocksPerSm<V>) dual_step_kernel(
   DualOp<V, true> op;
   op.sc = read_scalars<V>(d.st, false);
   const int cur = op.sc.cur, nxt = cur ^ 1;
-  op.prm = prm;
-  op.b = v.b; op.sense = d.sense;
-  op.axc = v.ax[cur]; op.yc = v.y[cur]; op.ybarc = v.ybar[cur];
-  op.S = v.S; op.invS = v.invS; op.GS = v.GS; op.p = v.p;
-  op.yn = v.y[nxt]; op.axn = v.ax[nxt]; op.ybarn = v.ybar[nxt];
-  op.acc[0] = op.acc[1] = op.acc[2] = op.acc[3] = V(0);
+  op.bind(v, prm, d.sense, cur);
   std::conditional_t<kHot, HotGather<V>, Gather<1, V>> g;
   g.x[0] = v.x[nxt];  // x+ written by the primal kernel
   g.n = d.n;

@@ -70,32 +70,79 @@ __device__ __noinline__ void ogd_entry(V* P, V* inv, V* G, V grad, int sched, V 
   ogd_entry_inline<V>(P, inv, G, grad, sched, alpha, floor, sqrt_gnorm);
 }
 
-template <class V, bool kInlineUpdate = false>
-struct PrimalOp {
-  const V *c, *l, *u, *xc, *xbarc;
-  V *T, *invT, *GT, *q, *xn, *xbarn;
+// A vector that a row operation works on, and the options it needs rarely.
+// The step kernels' are kernel arguments, that is constants.  The batched
+// kernel's are a member's and are in shared memory: they are read from there at
+// each use (a volatile load); held in registers, ten pointers and the options
+// more than the step kernels have, they spilled.
+template <class V, bool kStep>
+struct VecPtr {
+  V* p;
+  __device__ __forceinline__ static VecPtr of(V* const& q) { return VecPtr{q}; }
+  __device__ __forceinline__ operator V*() const { return p; }
+};
+template <class V>
+struct VecPtr<V, false> {
+  V* const* at;
+  __device__ __forceinline__ static VecPtr of(V* const& q) { return VecPtr{&q}; }
+  __device__ __forceinline__ operator V*() const { return *const_cast<V* const volatile*>(at); }
+};
+template <bool kStep>
+struct RowOptions {
   Params prm;
+  __device__ __forceinline__ static RowOptions of(const Params& q) { return RowOptions{q}; }
+  __device__ __forceinline__ const Params& get() const { return prm; }
+};
+template <>
+struct RowOptions<false> {
+  const Params* prm;
+  __device__ __forceinline__ static RowOptions of(const Params& q) { return RowOptions{&q}; }
+  __device__ __forceinline__ const Params& get() const { return *prm; }
+};
+
+template <class V, bool kStep>
+__device__ __forceinline__ void update_entry(V* P, V* inv, V* G, V grad, const Params& prm, V sqrt_gnorm) {
+  if (kStep) ogd_entry_inline<V>(P, inv, G, grad, prm.sched, (V)prm.alpha, (V)prm.floor, sqrt_gnorm);
+  else ogd_entry<V>(P, inv, G, grad, prm.sched, (V)prm.alpha, (V)prm.floor, sqrt_gnorm);
+}
+
+template <class V, bool kStep = false>
+struct PrimalOp {
+  using Ptr = VecPtr<V, kStep>;
+  Ptr c, l, u, xc, xbarc, T, invT, GT, q, xn, xbarn;
+  RowOptions<kStep> options;
+  int mode;
   StepScalars<V> sc;
   V acc[3];  // sum dx^2 / T, ||g||^2, sum q^2 (per thread; combined across threads in FP64)
   V pT, piT, pc, px, pl, pu, pxb;  // operands of the row being processed, loaded early
 
+  // the vectors of v, from half cur of the double buffers to the other
+  __device__ __forceinline__ void bind(const Vecs<V>& v, const Params& prm, int cur) {
+    c = Ptr::of(v.c); l = Ptr::of(v.l); u = Ptr::of(v.u);
+    xc = Ptr::of(v.x[cur]); xbarc = Ptr::of(v.xbar[cur]);
+    T = Ptr::of(v.T); invT = Ptr::of(v.invT); GT = Ptr::of(v.GT); q = Ptr::of(v.q);
+    xn = Ptr::of(v.x[cur ^ 1]); xbarn = Ptr::of(v.xbar[cur ^ 1]);
+    options = RowOptions<kStep>::of(prm);
+    mode = prm.mode;
+    acc[0] = acc[1] = acc[2] = V(0);
+  }
+
   __device__ __forceinline__ void prefetch(int j) {
-    pT = T[j];
-    piT = invT[j];
-    pc = __ldg(c + j);
-    px = xc[j];
-    pl = __ldg(l + j);
-    pu = __ldg(u + j);
-    if (prm.mode == kPdlp) pxb = xbarc[j];
+    pT = ((V*)T)[j];
+    piT = ((V*)invT)[j];
+    pc = __ldg((V*)c + j);
+    px = ((V*)xc)[j];
+    pl = __ldg((V*)l + j);
+    pu = __ldg((V*)u + j);
+    if (mode == kPdlp) pxb = ((V*)xbarc)[j];
   }
 
   __device__ __forceinline__ void row(int j, const V (&s)[1]) {
     V Tj = pT, iT = piT;
     if (sc.pend) {  // pending online update of T_j (rare: once every phi accepted steps)
-      if (kInlineUpdate) ogd_entry_inline<V>(T + j, invT + j, GT + j, sc.up_scale * q[j], prm.sched, (V)prm.alpha, (V)prm.floor, sc.sqrt_gnorm);
-      else ogd_entry<V>(T + j, invT + j, GT + j, sc.up_scale * q[j], prm.sched, (V)prm.alpha, (V)prm.floor, sc.sqrt_gnorm);
-      Tj = T[j];
-      iT = invT[j];
+      update_entry<V, kStep>((V*)T + j, (V*)invT + j, (V*)GT + j, sc.up_scale * ((V*)q)[j], options.get(), sc.sqrt_gnorm);
+      Tj = ((V*)T)[j];
+      iT = ((V*)invT)[j];
     }
     const V g = pc - s[0];
     const V x0 = px;
@@ -103,48 +150,59 @@ struct PrimalOp {
     const V lo = pl, hi = pu;
     const auto kx = ord_key(xh), kl = ord_key(lo), kh = ord_key(hi);
     const V x1 = clamp_keys(xh, kx, lo, kl, hi, kh);
-    xn[j] = x1;
-    if (prm.mode == kPdlp) xbarn[j] = pxb + sc.eta * x1;
+    ((V*)xn)[j] = x1;
+    if (mode == kPdlp) ((V*)xbarn)[j] = pxb + sc.eta * x1;
     const V dx = x1 - x0;
     acc[0] += dx * dx * iT;
     if (sc.collect) {
       const V gi = (kx >= kl && kx <= kh) ? g : V(0);
       const V qj = gi * g;
-      q[j] = qj;
+      ((V*)q)[j] = qj;
       acc[1] += g * g;
       acc[2] += qj * qj;
     }
   }
 };
 
-template <class V, bool kInlineUpdate = false>
+template <class V, bool kStep = false>
 struct DualOp {
-  const V *b, *axc, *yc, *ybarc;
+  using Ptr = VecPtr<V, kStep>;
+  Ptr b, axc, yc, ybarc, S, invS, GS, p, yn, axn, ybarn;
   const uint8_t* sense;
-  V *S, *invS, *GS, *p, *yn, *axn, *ybarn;
-  Params prm;
+  RowOptions<kStep> options;
+  int mode;
   StepScalars<V> sc;
   V acc[4];  // sum dy^2 / Sigma, dy . A dx, ||b - A x||^2, sum p^2
   V pS, piS, pa0, pb, py, pyb;  // operands of the row being processed, loaded early
   uint8_t psn;
 
+  __device__ __forceinline__ void bind(const Vecs<V>& v, const Params& prm, const uint8_t* row_sense, int cur) {
+    b = Ptr::of(v.b);
+    sense = row_sense;
+    axc = Ptr::of(v.ax[cur]); yc = Ptr::of(v.y[cur]); ybarc = Ptr::of(v.ybar[cur]);
+    S = Ptr::of(v.S); invS = Ptr::of(v.invS); GS = Ptr::of(v.GS); p = Ptr::of(v.p);
+    yn = Ptr::of(v.y[cur ^ 1]); axn = Ptr::of(v.ax[cur ^ 1]); ybarn = Ptr::of(v.ybar[cur ^ 1]);
+    options = RowOptions<kStep>::of(prm);
+    mode = prm.mode;
+    acc[0] = acc[1] = acc[2] = acc[3] = V(0);
+  }
+
   __device__ __forceinline__ void prefetch(int i) {
-    pS = S[i];
-    piS = invS[i];
-    pa0 = axc[i];
-    pb = __ldg(b + i);
-    py = yc[i];
+    pS = ((V*)S)[i];
+    piS = ((V*)invS)[i];
+    pa0 = ((V*)axc)[i];
+    pb = __ldg((V*)b + i);
+    py = ((V*)yc)[i];
     psn = __ldg(sense + i);
-    if (prm.mode == kPdlp) pyb = ybarc[i];
+    if (mode == kPdlp) pyb = ((V*)ybarc)[i];
   }
 
   __device__ __forceinline__ void row(int i, const V (&s)[1]) {
     V Si = pS, iS = piS;
     if (sc.pend) {
-      if (kInlineUpdate) ogd_entry_inline<V>(S + i, invS + i, GS + i, sc.up_scale * p[i], prm.sched, (V)prm.alpha, (V)prm.floor, sc.sqrt_gnorm);
-      else ogd_entry<V>(S + i, invS + i, GS + i, sc.up_scale * p[i], prm.sched, (V)prm.alpha, (V)prm.floor, sc.sqrt_gnorm);
-      Si = S[i];
-      iS = invS[i];
+      update_entry<V, kStep>((V*)S + i, (V*)invS + i, (V*)GS + i, sc.up_scale * ((V*)p)[i], options.get(), sc.sqrt_gnorm);
+      Si = ((V*)S)[i];
+      iS = ((V*)invS)[i];
     }
     const V a1 = s[0];
     const V a0 = pa0;
@@ -157,16 +215,16 @@ struct DualOp {
     // <= rows keep y <= 0, >= rows keep y >= 0, equality rows are free
     const bool outside = (sn == kLe && ky > 0) || (sn == kGe && ky < 0);
     const V y1 = outside ? V(0) : yh;
-    yn[i] = y1;
-    axn[i] = a1;
-    if (prm.mode == kPdlp) ybarn[i] = pyb + sc.eta * y1;
+    ((V*)yn)[i] = y1;
+    ((V*)axn)[i] = a1;
+    if (mode == kPdlp) ((V*)ybarn)[i] = pyb + sc.eta * y1;
     const V dy = y1 - y0;
     acc[0] += dy * dy * iS;
     acc[1] += dy * (a1 - a0);
     if (sc.collect) {
       const V res = bi - a0;
       const V pi = outside ? V(0) : res * r;
-      p[i] = pi;
+      ((V*)p)[i] = pi;
       acc[2] += res * res;
       acc[3] += pi * pi;
     }
