@@ -281,10 +281,15 @@ int preprocess(lp_problem* p) {
   double* red = d.work + m + n;  // reduction scratch [1 + 1024]
   launch_fill(d.dr, 1.0, m, s);
   launch_fill(d.dc, 1.0, n, s);
-  auto apply = [&]() { launch_ruiz_apply(d, p->ruiz[0], p->ruiz[1], fr, fc, s); };
-  for (int r = 0; r < p->opt.ruiz_iters; ++r) {
-    launch_ruiz_norms(d, p->ruiz[0], p->ruiz[1], fr, fc, s);
-    apply();
+  // norms of one round into one pair of buffers while the factors of the round before are in the other
+  double* nr[2] = {fr, d.f64.p};
+  double* nc[2] = {fc, d.f64.q};
+  const int rounds = p->opt.ruiz_iters;
+  if (rounds > 0) launch_ruiz_norms(d, p->ruiz[0], p->ruiz[1], nr[0], nc[0], s);
+  for (int r = 0; r < rounds; ++r) {
+    const int k = r & 1;
+    const bool more = r + 1 < rounds;
+    launch_ruiz_apply(d, p->ruiz[0], p->ruiz[1], nr[k], nc[k], more ? nr[k ^ 1] : nullptr, more ? nc[k ^ 1] : nullptr, s);
   }
   if (p->opt.mode == LP_MODE_PDLP) {
     launch_row_powsum(d.A, m, p->ruiz[0].nlong, p->ruiz[0].split, p->opt.pc_beta, 0, fr, s);
@@ -293,7 +298,7 @@ int preprocess(lp_problem* p) {
     launch_row_powsum(d.A, m, p->ruiz[0].nlong, p->ruiz[0].split, 2.0, 1, fr, s);
     launch_row_powsum(d.At, n, p->ruiz[1].nlong, p->ruiz[1].split, 2.0, 1, fc, s);
   }
-  apply();
+  launch_ruiz_apply(d, p->ruiz[0], p->ruiz[1], fr, fc, nullptr, nullptr, s);
   CK(cudaGetLastError());
   int rc = LP_OK;
   // norms of the caller's b and c (still unscaled), then rescale the vectors

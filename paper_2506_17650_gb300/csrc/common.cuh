@@ -506,7 +506,8 @@ void launch_fill(double* v, double val, long long n, cudaStream_t s);
 // longest first; rows from split on have at most 32 entries):
 //   norms: fr = row infinity norms of A, fc = those of A^T (columns of A);
 //   apply: f <- f > 0 ? 1/sqrt(f) : 1 for fr and fc, dr *= fr, dc *= fc, and
-//          every entry a_ij <- (a_ij fr_i) fc_j in both copies.
+//          every entry a_ij <- (a_ij fr_i) fc_j in both copies; with nr and nc
+//          given, also the norms of the scaled rows into them.
 // How the Ruiz kernels cut the rows of one matrix: rows [0, nlong) (the
 // whole-block rows) in chunks of kRuizChunk entries, one warp each
 // (chunk_pre: device prefix of their chunk counts, nlong + 1 entries, nchunks
@@ -520,7 +521,8 @@ struct RuizSplit {
   const int* chunk_pre;
 };
 void launch_ruiz_norms(const Dev& d, const RuizSplit& a, const RuizSplit& at, double* fr, double* fc, cudaStream_t s);
-void launch_ruiz_apply(const Dev& d, const RuizSplit& a, const RuizSplit& at, double* fr, double* fc, cudaStream_t s);
+void launch_ruiz_apply(const Dev& d, const RuizSplit& a, const RuizSplit& at, double* fr, double* fc, double* nr, double* nc,
+                       cudaStream_t s);
 // out[r] = sum over row r of |a|^beta (optionally its square root); rows [0, nlong) are the whole-block
 // rows, rows [split, rows) those of at most 32 entries
 void launch_row_powsum(const Csr& M, int rows, int nlong, int split, double beta, int square_root, double* out,

