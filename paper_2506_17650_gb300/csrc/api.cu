@@ -30,6 +30,10 @@ void launch_scatter_perm(double* out, const double* a, const double* f, const in
 void launch_gather_perm(double* out, const double* a, const int* perm, int n, cudaStream_t s);
 void launch_result(const Dev& d, bool fp32, double* x, double* y, const int* prow, const int* pcol, cudaStream_t s);
 void launch_begin_solve(DevState* st, double tol, cudaStream_t s);
+// noalloc.cu
+size_t power_norm_state_bytes();
+cudaError_t power_norm(int m, int n, long long nnz, const Csr& A, const Csr& At, int iters, const int* perm,
+                       bool in_order, double* w, double* t, double* part, void* state, cudaStream_t s, double* norm);
 void row_kernel_blocks_per_sm(int* primal, int* dual, int* primal32, int* dual32);
 }  // namespace lpop
 
@@ -44,6 +48,7 @@ struct lp_problem {
   lp_options opt{};
   int device = 0;
   int sms = 0;
+  int longest = 0;  // entries of the longest row of A or A^T (at least; 2048 when none is longer)
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   Dev d{};
@@ -271,6 +276,11 @@ double read_scalar(lp_problem* p, const double* dptr, int* rc) {
   return p->h_scratch[0];
 }
 
+// Longest row for which the power iteration of lp_create runs as two kernels a
+// round with a warp per long row; with longer ones it takes the row classes of
+// the layout (a block per long row) and five launches.
+constexpr int kPowerMaxRow = 8192;
+
 int preprocess(lp_problem* p) {
   NvtxRange range("lpop preprocess");
   Dev& d = p->d;
@@ -333,7 +343,11 @@ int preprocess(lp_problem* p) {
     double* t = d.f64.ax_avg;  // [m]
     double* w = fc;        // [n]
     p->norm_est = 0.0;
-    if (p->nnz > 0) {
+    if (p->nnz > 0 && p->longest <= kPowerMaxRow) {
+      double nw = 0.0;
+      CK(power_norm(m, n, p->nnz, d.A, d.At, p->opt.power_iters, p->d_pcol, true, w, t, red, red + 1024, s, &nw));
+      p->norm_est = nw > 0.0 && std::isfinite(nw) ? std::sqrt(nw) : 0.0;
+    } else if (p->nnz > 0) {
       launch_fill(v, 1.0 / std::sqrt((double)n), n, s);
       bool restarted = false;
       for (int it = 0; it < p->opt.power_iters; ++it) {
@@ -550,6 +564,9 @@ int upload(lp_problem* p, int m, int n, long long nz, const int64_t* row_ptr, co
       if (4LL * entries[1] >= nz) d.hot32 = hot32;
     }
   }
+  p->longest = 2048;
+  for (const std::vector<int>* head : {&lay.A_head, &lay.At_head})
+    if (head->size() > 1) p->longest = std::max(p->longest, (*head)[1] - (*head)[0]);
   for (int which = 0; which < 2; ++which) {  // Ruiz units: whole-block rows in chunks, then warp and thread rows
     const std::vector<int>& head = which ? lay.At_head : lay.A_head;
     RuizSplit& rs = p->ruiz[which];

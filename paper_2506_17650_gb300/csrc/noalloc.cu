@@ -54,10 +54,10 @@ int scratch_address(int dev, double** out) {
   return LP_OK;
 }
 
-// v[j] = scale * (+-1 from SplitMix64 of j): the power iteration's second start direction.
-__global__ void splitmix_fill_kernel(double* v, int n, double scale) {
+// v[j] = scale * (+-1 from SplitMix64 of j, or of perm[j]): the power iteration's second start direction.
+__global__ void splitmix_fill_kernel(double* v, int n, double scale, const int* perm) {
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
-    v[j] = scale * splitmix_sign((unsigned long long)j);
+    v[j] = scale * splitmix_sign((unsigned long long)(perm ? perm[j] : j));
 }
 
 // Scalars of the iteration, after the partial sums.
@@ -163,17 +163,54 @@ __global__ void __launch_bounds__(kBlock) norm_rows_kernel(int rows, const int* 
 
 template <bool kNorm>
 void launch_norm_rows(int rows, const int* rp, const int* ci, const double* val, const double* x, double* y,
-                      NormState* st, double* part, double mean, cudaStream_t s) {
-  const int W = mean <= 8.0 ? 2 : (mean <= 32.0 ? 4 : (mean <= 128.0 ? 8 : 32));
+                      NormState* st, double* part, double mean, bool one_lane, cudaStream_t s) {
+  const int W = one_lane && mean <= 16.0 ? 1 : mean <= 8.0 ? 2 : (mean <= 32.0 ? 4 : (mean <= 128.0 ? 8 : 32));
   const long long warps = ((long long)rows * W + 31) / 32;
   const int grid = (int)std::min<long long>(912, (warps + kBlock / 32 - 1) / (kBlock / 32));  // six blocks on each of 152 SMs
-  if (W == 2) launch_pdl(norm_rows_kernel<2, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
+  if (W == 1) launch_pdl(norm_rows_kernel<1, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
+  else if (W == 2) launch_pdl(norm_rows_kernel<2, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
   else if (W == 4) launch_pdl(norm_rows_kernel<4, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
   else if (W == 8) launch_pdl(norm_rows_kernel<8, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
   else launch_pdl(norm_rows_kernel<32, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
 }
 
 }  // namespace
+
+size_t power_norm_state_bytes() { return sizeof(NormState); }
+
+// ||w|| of the last of `iters` rounds w = A^T A w / ||w|| from the all-ones
+// direction, or (a zero first product: every row of A sums to zero) from the
+// SplitMix64 sign direction.  w [n], t [m], part [1024], state: device scratch.
+// in_order: short rows are summed by one lane, as one chain of FMAs (whether
+// rows that sum to zero give exactly zero depends on that, and with it the
+// start direction).
+cudaError_t power_norm(int m, int n, long long nnz, const Csr& A, const Csr& At, int iters, const int* perm,
+                       bool in_order, double* w, double* t, double* part, void* state, cudaStream_t s, double* norm) {
+  NormState* st = static_cast<NormState*>(state);
+  NormState h{};
+  for (int start = 0; start < 2; ++start) {
+    const double one = 1.0 / std::sqrt((double)n);
+    if (start == 0) {
+      launch_fill(w, one, n, s);
+    } else {
+      const int g = (n + kBlock - 1) / kBlock;
+      splitmix_fill_kernel<<<g < 1024 ? g : 1024, kBlock, 0, s>>>(w, n, one, perm);
+    }
+    norm_init_kernel<<<1, 1, 0, s>>>(st);
+    for (int it = 0; it < iters; ++it) {
+      launch_norm_rows<false>(m, A.rp, A.ci, A.v, w, t, st, part, (double)nnz / m, in_order, s);
+      launch_norm_rows<true>(n, At.rp, At.ci, At.v, t, w, st, part, (double)nnz / n, in_order, s);
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return e;
+    if (h.first != 0.0) break;
+  }
+  *norm = h.norm;
+  return cudaSuccess;
+}
+
 }  // namespace lpop
 
 using namespace lpop;
@@ -199,39 +236,15 @@ extern "C" int lp_power_norm_noalloc(int32_t m, int32_t n, const int32_t* a_row_
   if (rc != LP_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // w (n) | t (m) | partial sums (1024); the scalars after the array's 2^20 doubles
-  double* w = scratch;
-  double* t = w + n;
-  double* part = t + m;
-  NormState* st = reinterpret_cast<NormState*>(scratch + kScratchDoubles);
   static_assert(sizeof(NormState) <= 8 * sizeof(double), "scalars after the array");
-
-  NormState h{};
   int nnz = 0;
   e = cudaMemcpyAsync(&nnz, a_row_ptr + m, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return fail(LP_ERR_CUDA, std::string("reading the matrix size failed: ") + cudaGetErrorString(e));
-  for (int start = 0; start < 2; ++start) {
-    const double one = 1.0 / std::sqrt((double)n);
-    if (start == 0) {
-      launch_fill(w, one, n, s);
-    } else {
-      splitmix_fill_kernel<<<(n + kBlock - 1) / kBlock < 1024 ? (n + kBlock - 1) / kBlock : 1024, kBlock, 0, s>>>(w, n, one);
-    }
-    norm_init_kernel<<<1, 1, 0, s>>>(st);
-    for (int it = 0; it < iters; ++it) {
-      launch_norm_rows<false>(m, a_row_ptr, a_col_idx, a_val, w, t, st, part, (double)nnz / m, s);
-      launch_norm_rows<true>(n, at_row_ptr, at_col_idx, at_val, t, w, st, part, (double)nnz / n, s);
-    }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(LP_ERR_CUDA, std::string("kernel launch failed: ") + cudaGetErrorString(e));
-    e = cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return fail(LP_ERR_CUDA, std::string("reading the result failed: ") + cudaGetErrorString(e));
-    // a zero first product (every row of A sums to zero): start again from
-    // the SplitMix64 sign direction, as lp_create does
-    if (h.first != 0.0) break;
-  }
-  const double nw = h.norm;
+  double nw = 0.0;
+  if (e == cudaSuccess)
+    e = power_norm(m, n, nnz, Csr{a_row_ptr, a_col_idx, a_val}, Csr{at_row_ptr, at_col_idx, at_val}, iters, nullptr, false,
+                   scratch, scratch + n, scratch + n + m, scratch + kScratchDoubles, s, &nw);
+  if (e != cudaSuccess) return fail(LP_ERR_CUDA, std::string("power iteration failed: ") + cudaGetErrorString(e));
   *norm_out = nw > 0.0 && std::isfinite(nw) ? std::sqrt(nw) : 0.0;
   return LP_OK;
 }
