@@ -1006,7 +1006,7 @@ const ResPlan* resident_plan(lp_problem* p, int* rc) {
       return LP_OK;
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t ib = h.items.size() * sizeof(ResItem), cb = h.cta.size() * sizeof(ResCta);
-    const size_t o1 = up(ib), o2 = o1 + up(cb), o3 = o2 + up(16 * (8 * (size_t)h.plan.G + 8));
+    const size_t o1 = up(ib), o2 = o1 + up(cb), o3 = o2 + up(16 * (8 * (size_t)h.plan.G + 8 + (size_t)h.plan.segs));
     const size_t o4 = o3 + up((size_t)(p->d.n + 2LL * p->d.m) * 2 * esize);
     if ((long long)(o4 + 256) > resident_bytes(p->d.m, p->d.n, p->nnz, esize)) return LP_OK;
     CK(cudaMemcpyAsync(R.block, h.items.data(), ib, cudaMemcpyHostToDevice, p->stream));
@@ -1017,6 +1017,7 @@ const ResPlan* resident_plan(lp_problem* p, int* rc) {
     h.plan.cta = reinterpret_cast<const ResCta*>(R.block + o1);
     h.plan.rec = reinterpret_cast<ulonglong2*>(R.block + o2);
     h.plan.ctl = h.plan.rec + 7 * h.plan.G;
+    h.plan.seg = h.plan.ctl + h.plan.G + 8;
     h.plan.gx = R.block + o3;
     h.plan.bar = reinterpret_cast<unsigned int*>(R.block + o4);
     R.plan = h.plan;

@@ -11,10 +11,12 @@
 // The sums over the CTAs travel the same way.
 //
 // Measured (64 attempts with their two checks, reset and result, FP64, against
-// the two-kernel path): 4,001 x 10,003 with 60k nonzeros 1,368 -> 709 us; 1,003
-// x 8,005 with 376k nonzeros in rows of up to 3,000: 1,918 -> 1,112 us; 50,000 x
-// 200,000 transportation, 400k nonzeros: 1,875 -> 1,293 us; 200 x 500 with 2.5k
-// nonzeros, 256 attempts in one CTA: 4,235 -> 1,849 us.
+// the two-kernel path): 4,001 x 10,003 with 60k nonzeros 1,368 -> 700 us; 1,003
+// x 8,005 with 376k nonzeros in rows of up to 3,000: 1,918 -> 946 us (1,112 with
+// rows of more than 2,048 entries summed by a whole CTA instead of in segments of
+// 512 by warps of all CTAs); 50,000 x 200,000 transportation, 400k nonzeros:
+// 1,875 -> 1,262 us; 200 x 500 with 2.5k nonzeros, 256 attempts in one CTA: 4,235
+// -> 1,815 us.
 #include "resident.hpp"
 
 #include <algorithm>
@@ -275,11 +277,10 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
   V* const s_vd = reinterpret_cast<V*>(s_raw + L.vd);
   V* const s_xp = reinterpret_cast<V*>(s_raw + L.xp);
   V* const s_xd = reinterpret_cast<V*>(s_raw + L.xd);
-  double* const s_wide = reinterpret_cast<double*>(s_raw + L.wide);
   double* const s_red = reinterpret_cast<double*>(s_raw + L.red);
   int* const s_cp = reinterpret_cast<int*>(s_raw + L.cp);
   int* const s_cd = reinterpret_cast<int*>(s_raw + L.cd);
-  int* const s_lrp = reinterpret_cast<int*>(s_raw + L.lrp);
+  int2* const s_lrp = reinterpret_cast<int2*>(s_raw + L.lrp);  // first entry, length
   int* const s_gp = reinterpret_cast<int*>(s_raw + L.gp);
   int* const s_gd = reinterpret_cast<int*>(s_raw + L.gd);
   ResItem* const s_it = reinterpret_cast<ResItem*>(s_raw + L.it);
@@ -330,6 +331,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
       const CsrT<V> M = P ? csr_at<V>(d) : csr_a<V>(d);
       V* sv = (P ? s_vp : s_vd) + I.ent;
       int* sc = (P ? s_cp : s_cd) + I.ent;
+      const bool far = kBars && (pl.far >> (P ? 0 : 1) & 1);
       if (I.kind == 0) {  // entry k of the slice's row t at 32 k + t
         if (lane < I.nrows) {
           const int e0 = M.rp[I.row0 + lane], len = M.rp[I.row0 + lane + 1] - e0;
@@ -341,19 +343,21 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
           }
         }
       } else {
-        const int e0 = M.rp[I.row0], e1 = M.rp[I.row0 + I.nrows];
+        const int e0 = M.rp[I.row0] + (I.kind == kSegKind ? I.len : 0);
+        const int e1 = I.kind == kSegKind ? e0 + I.nrows : I.kind == kOwnKind ? e0 : M.rp[I.row0 + I.nrows];
+        if (!far) {
 #pragma unroll 2
-        for (int k = e0 + lane; k < e1; k += 32) {
-          sc[k - e0] = M.ci[k];
-          sv[k - e0] = M.v[k];
+          for (int k = e0 + lane; k < e1; k += 32) {
+            sc[k - e0] = M.ci[k];
+            sv[k - e0] = M.v[k];
+          }
         }
-        const int q = (P ? 0 : C.nlp + 1) + I.len;
-        // (a row's end is the next long row's start; the last one writes its own)
-        const int ends = I.nrows + (I.len + I.nrows == (P ? C.nlp : C.nld) ? 1 : 0);
-#pragma unroll 1
-        for (int r = lane; r < ends; r += 32) s_lrp[q + r] = I.ent + M.rp[I.row0 + r] - e0;
+        if (I.kind <= 32 && lane < I.nrows) {
+          const int q = (P ? 0 : C.nlp) + I.len + lane, first = M.rp[I.row0 + lane];
+          s_lrp[q] = int2{far ? first : I.ent + first - e0, M.rp[I.row0 + lane + 1] - first};
+        }
       }
-      if (lane < I.nrows) {
+      if (I.kind != kSegKind && lane < I.nrows) {
         const int row = I.row0 + lane, t = I.vec + lane;
         if (P) {
           s_gp[t] = row;
@@ -396,58 +400,56 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
   }
   __syncthreads();
 
-  // One side's row sums, by warps w0, w0 + 1, ...: into sum[local row], but a
-  // CTA-wide row's into the warps' parts in s_wide (wide_total adds them).
-  auto row_sums = [&](const ResItem* it, int n, int nwide, const V* sv, const int* sc, const int* lrp,
-                      const uint8_t* lens, const ResGather<V, kKind>& g, V* sum, int w0) {
+  // One side's row sums, by warps w0, w0 + 1, ...: into sum[local row].
+  auto row_sums = [&](const ResItem* it, int n, const V* sv, const int* sc, const int2* lrp, const uint8_t* lens,
+                      const CsrT<V>* far, const ResGather<V, kKind>& g, V* sum, int w0) {
     bool ok = true;
-    const int me = warp - w0, nw = kResWarps - w0;
 #pragma unroll 1
-    for (int k = 0;; ++k) {
-      const int i = k < nwide ? k : nwide + (k - nwide) * nw + me;
-      if (i >= n) break;
+    for (int i = warp - w0; i < n; i += kResWarps - w0) {
       const ResItem& I = it[i];
+      if (!kSolo && I.kind == kOwnKind) {  // the segments' sums, in segment order over the lanes
+        double t;
+        ok = rec_sum(pl.seg + I.ent, I.len, g.seq, &t) && ok;
+        if (lane == 0) sum[I.vec] = (V)t;
+        continue;
+      }
       int off, count, most, step = 32;
       if (I.kind == 0) {
         off = I.ent + lane;
         count = lane < I.nrows ? lens[I.vec + lane] : 0;
         most = I.len;
+      } else if (!kSolo && I.kind == kSegKind) {
+        off = I.ent + lane;
+        count = (I.nrows - lane + 31) >> 5;
+        most = (I.nrows + 31) >> 5;
       } else {
-        const bool wide = I.kind == kResThreads;
-        const int lg = wide ? 5 : 31 - __clz(I.kind);
-        step = wide ? 32 * nw : I.kind;
-        const int l = wide ? 32 * me + lane : lane & (I.kind - 1);
-        const int r = wide ? 0 : lane >> lg;
+        const int lg = 31 - __clz(I.kind);
+        step = I.kind;
+        const int l = lane & (step - 1), r = lane >> lg;
         const bool has = r < I.nrows;
-        off = lrp[I.len + (has ? r : 0)] + l;
-        const int left = has ? lrp[I.len + r + 1] - off + step - 1 : 0;
-        count = wide ? left / step : left >> lg;
+        const int2 e = lrp[I.len + (has ? r : 0)];
+        off = e.x + l;
+        count = has ? (max(e.y - l, 0) + step - 1) >> lg : 0;
         most = __reduce_max_sync(0xffffffffu, count);
       }
-      V s = res_dot(sv + off, sc + off, count, most, step, g, &ok);
+      V s;
+      if (kBars && far) s = res_dot(far->v + off, far->ci + off, count, most, step, g, &ok);
+      else s = res_dot(sv + off, sc + off, count, most, step, g, &ok);
       if (I.kind == 0) {
         if (lane < I.nrows) sum[I.vec + lane] = s;
-      } else if (I.kind <= 32) {
+      } else if (!kSolo && I.kind == kSegKind) {
+        const double w = lane_sum((double)s);
+        if (lane == 0) ResElt<double>::put(pl.seg + I.vec, w, g.seq);
+      } else {
+        const int lg = 31 - __clz(step);
 #pragma unroll 1
         for (int o = step / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, step);
-        const int lg = 31 - __clz(step);
         if ((lane & (step - 1)) == 0 && (lane >> lg) < I.nrows) sum[I.vec + (lane >> lg)] = s;
-      } else {
-        const double w = lane_sum((double)s);
-        if (lane == 0) s_wide[i * kResWarps + warp] = w;
       }
     }
     if (!kSolo && !ok) s_ok = 0;
   };
-  auto wide_total = [&](int i, int w0) {
-    double w = 0.0;
-#pragma unroll 1
-    for (int k = w0; k < kResWarps; ++k) w += s_wide[i * kResWarps + k];
-    return (V)w;
-  };
-  int nwp = 0, nwd = 0;  // CTA-wide rows: the first items of a side
-  while (nwp < np && s_it[nwp].kind == kResThreads) ++nwp;
-  while (nwd < nd && s_it[np + nwd].kind == kResThreads) ++nwd;
+  const CsrT<V> far_a = csr_a<V>(d), far_at = csr_at<V>(d);
   const int wp = min(kResWarps, (C.rp + 31) / 32), wd = min(kResWarps, (C.rd + 31) / 32);  // warps with rows
 
   unsigned int target = arrived + pl.G;  // arrivals of all CTAs so far
@@ -514,7 +516,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
       const StepScalars<V> sd = read_scalars<V>(&s_st, false);
       V* const axc = dax + cur * pl.rd;
       V* const axn = dax + nxt * pl.rd;
-      row_sums(s_it + np, nd, nwd, s_vd, s_cd, s_lrp + C.nlp + 1, s_lend, ResGather<V, kKind>{kSolo ? xn : v.x[nxt], gxw, seq, d.n, d.bad_gathers}, axn, 0);
+      row_sums(s_it + np, nd, s_vd, s_cd, s_lrp + C.nlp, s_lend, pl.far & 2 ? &far_a : nullptr,
+               ResGather<V, kKind>{kSolo ? xn : v.x[nxt], gxw, seq, d.n, d.bad_gathers}, axn, 0);
       __syncthreads();
       V accd[4] = {V(0), V(0), V(0), V(0)};
 #pragma unroll 1
@@ -526,9 +529,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
           v.S[row] = dS[t];
           v.invS[row] = diS[t];
         }
-        V a1;
-        if (t < nwd) axn[t] = a1 = wide_total(t, 0);
-        else a1 = axn[t];
+        const V a1 = axn[t];
         const V a0 = axc[t], bi = db[t], y0 = yc[t];
         const V r = bi - (V(2) * a1 - a0);
         const V yh = y0 + sd.step * dS[t] * r;
@@ -626,7 +627,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
         }
         rows_sync();
       }
-      row_sums(s_it, np, nwp, s_vp, s_cp, s_lrp, s_lenp,
+      row_sums(s_it, np, s_vp, s_cp, s_lrp, s_lenp, pl.far & 1 ? &far_at : nullptr,
                ResGather<V, kKind>{kSolo ? yn : v.y[nxt], gyw + (size_t)nxt * d.m, seq, d.m, d.bad_gathers}, psum + nxt * pl.rp, kCtlWarps);
       if (avg) {  // the last accepted attempt's terms of the averages
         const int t0 = tid - 32 * kCtlWarps, step = kResThreads - 32 * kCtlWarps;
@@ -640,10 +641,6 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
     if (!kSolo && !s_ok) {
       if (tid == 0) d.st->fault = 1;
       return;
-    }
-    if (nwp > 0) {
-      if (tid < nwp) psum[nxt * pl.rp + tid] = wide_total(tid, kCtlWarps);
-      __syncthreads();
     }
     if (kBars && a >= 0) target += pl.G;
     avg_eta = sp.eta;
@@ -699,7 +696,8 @@ const void* resident_fn(bool fp32, int kind) {
 // against 1,348).
 constexpr int kWordsMaxRow = 128;
 int resident_kind(const ResPlan& pl) {
-  return pl.G == 1 ? kSoloKind : (pl.longest <= kWordsMaxRow ? kWordsKind : kBarriersKind);
+  if (pl.G == 1) return kSoloKind;
+  return pl.longest <= kWordsMaxRow && !pl.far ? kWordsKind : kBarriersKind;
 }
 
 }  // namespace

@@ -11,7 +11,9 @@
 // per attempt only x+ and y+ travel (through L2), between grid-wide barriers,
 // and every CTA sums the G records and runs the step control on its own copy
 // of the state.  A problem that fits in one SM takes a single CTA and no grid
-// barrier.  resident.cu has the measured times and the choice of G.
+// barrier.  Where the vectors fit but not both copies of the matrix, one or both
+// copies are read from global memory (L2) in each attempt.  resident.cu and
+// resident_plan.cpp have the measured times and the choices.
 #pragma once
 
 #include "common.cuh"

@@ -17,8 +17,10 @@ namespace lpop {
 constexpr int kResThreads = 512;
 constexpr int kResWarps = kResThreads / 32;
 constexpr int kResMaxCtas = 160;   // records and tables are sized for this many
-constexpr int kResWide = 16;       // rows of a CTA that all its warps sum together, at most
-constexpr int kResMaxRow = 8192;   // longest row (entries) of a resident problem
+constexpr int kResSeg = 512;       // entries of a segment of a long row (G > 1)
+constexpr int kResMaxSegs = 160;   // segments of a row, at most
+constexpr int kSegKind = 64;       // kinds of items (1, 2, ... 32: lanes per row)
+constexpr int kOwnKind = 65;
 
 // A warp's work: `nrows` consecutive rows from row0 (bin order), local rows
 // from `vec`, entries from `ent` in the CTA's entry arrays.  kind 0: a slice
@@ -26,9 +28,14 @@ constexpr int kResMaxRow = 8192;   // longest row (entries) of a resident proble
 // t at ent + 32 k + t, `len` the longest row; neighbours in bin order have
 // similar lengths, so few lanes idle, and a small matrix needs one slice where
 // slices of one exact length would take many).  kind 2..32: CSR rows of kind
-// lanes each; kind kResThreads: one CSR row summed by the whole CTA.  For
-// those, `len` is the row's index among the CTA's long rows, which are its
-// first local rows.
+// lanes each; `len` is then the row's index among the CTA's long rows, which
+// are its first local rows.  A row of more than kResSeg entries is cut: its
+// segments (kind kSegKind: `nrows` entries of row row0 from entry `len` on) are
+// dealt to warps of all CTAs and leave their sums in words `vec`; the CTA that
+// has the row adds them up (kind kOwnKind: words ent, ent + 1, ... `len` of
+// them).  A segment of a side whose entries stay in global memory has its place
+// in the CSR arrays in ent; other items of such a side are all of CSR rows, and
+// their ent is unused.
 struct ResItem {
   int row0, nrows, len, kind;
   int ent, vec;
@@ -46,10 +53,13 @@ struct ResPlan {
   const ResCta* cta;
   ulonglong2* rec;    // [7 * G] records of an attempt, field by field
   ulonglong2* ctl;    // [8 * (G / 8 + 1)] result of the step control, a line for each eight CTAs
+  ulonglong2* seg;    // words of the segments: those of A^T, then those of A
   void* gx;           // words of x+ [n], then of y+ [2][m]
   unsigned int* bar;  // arrivals, number of the last attempt, start decision, arrivals before this launch
   int G;
   int ep, ed, rp, rd, lp, ld, it;  // entries, rows, long rows of A^T / A; items of both
+  int far;                         // 1: the entries of A^T, 2: those of A are read from the global CSR arrays
+  int segs, segs_d;                // segments of both sides, and of A
   int longest;                     // entries of the longest row of A or A^T
   int smem;                        // dynamic shared memory, bytes
 };
@@ -58,10 +68,9 @@ struct ResPlan {
 struct ResLayout {
   int vp, vd;    // values of A^T / A entries
   int xp, xd;    // ten vectors per A^T row, eight per A row
-  int wide;      // warps' sums of the CTA-wide rows
   int red;       // block sums: four fields of kResThreads doubles
   int cp, cd;    // column indices
-  int lrp;       // first entry of the long rows (A^T rows, then A rows)
+  int lrp;       // first entry and length of the long rows (A^T rows, then A rows)
   int gp, gd;    // global rows
   int it, sense;
   int lenp, lend;  // lengths of the slices' rows
@@ -77,11 +86,10 @@ LPOP_HD inline ResLayout res_layout(const ResPlan& p, int esize) {
   L.vd = o; o += up16(p.ed * esize);
   L.xp = o; o += up16(10 * p.rp * esize);
   L.xd = o; o += up16(8 * p.rd * esize);
-  L.wide = o; o += kResWide * kResWarps * 8;
   L.red = o; o += 4 * kResThreads * 8;
   L.cp = o; o += up16(p.ep * 4);
   L.cd = o; o += up16(p.ed * 4);
-  L.lrp = o; o += up16((p.lp + p.ld + 2) * 4);
+  L.lrp = o; o += up16((p.lp + p.ld) * 8);
   L.gp = o; o += up16(p.rp * 4);
   L.gd = o; o += up16(p.rd * 4);
   L.it = o; o += up16(p.it * (int)sizeof(ResItem));

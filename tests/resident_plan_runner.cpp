@@ -38,7 +38,7 @@ int main(int argc, char** argv) {
   const ResLayout L = res_layout(out.plan, esize);
   const int64_t head[] = {ok, (int64_t)out.items.size(), (int64_t)out.cta.size(), out.plan.G, out.plan.ep, out.plan.ed,
                           out.plan.rp, out.plan.rd, out.plan.lp, out.plan.ld, out.plan.it, out.plan.smem, L.total,
-                          resident_bytes(lay.m, lay.n, lay.nnz, esize)};
+                          resident_bytes(lay.m, lay.n, lay.nnz, esize), out.plan.far};
   std::fwrite(head, 8, sizeof(head) / 8, f);
   for (const ResItem& i : out.items) {
     const int64_t r[] = {i.row0, i.nrows, i.len, i.kind, i.ent, i.vec};

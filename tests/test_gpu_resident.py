@@ -1,6 +1,7 @@
 """Resident check periods (csrc/resident.cu): problems held in the shared memory
 of one CTA, of several CTAs that exchange words, and of several with grid
-barriers (a row or column of more than 128 entries).
+barriers (a row or column of more than 128 entries), with long rows cut into
+segments and with one side's entries in global memory.
 
 * 40 attempts (online updates included) against the oracle within 1e-10 and
   against the two-kernel path (which kernel timing selects) within 1e-10: the
@@ -28,6 +29,10 @@ CASES = {
     "words": (lambda: lpgen.batch_member(9, 701, 1_753), dict(alpha=1e-3, phi=5)),
     "words_transport": (lambda: lpgen.transport(1, 1_501, 1_499, 12_007), dict(alpha=1e-4, phi=20)),
     "barriers_wide_rows": (lambda: lpgen.row_length_mix(2), dict(alpha=1e-3, phi=7)),
+    # a row of 4,097..11,000 entries of A and of A^T: segments on both sides
+    "barriers_segments": (lambda: lpgen.long_rows(2), dict(alpha=1e-3, phi=20)),
+    # too large for shared memory with both copies of the matrix: one side read from global memory
+    "one_side_far": (lambda: lpgen.powerlaw(2, 50_000, 125_000, 800_000), dict(alpha=1e-6, phi=20)),
     "barriers_powerlaw": (lambda: lpgen.powerlaw(1, 6_001, 15_003, 90_000, dmax=5_000), dict(alpha=1e-6, phi=20)),
 }
 MODE = {"plain": lpop.LP_MODE_PLAIN, "pdlp": lpop.LP_MODE_PDLP}
