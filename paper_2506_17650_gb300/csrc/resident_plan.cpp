@@ -108,9 +108,10 @@ struct Deal {
 
 // Among items of one cost the CTAs that took one stand in line in the order in
 // which they took it, so the next is the first of that line or of the CTAs that
-// have not had one: no heap is needed, and the plan of a power-law
-// LP of 1M entries (three deals of 16,000 to 24,000 items) takes a tenth of the
-// time that sorting the items and dealing them through a heap took.
+// have not had one: no heap is needed.  The first solve pays for the plan (a
+// power-law LP of 1M entries: three deals of 16,000 to 24,000 items); with the
+// items sorted and dealt through a heap it took 7,476 us, now 2,828 (a later
+// solve 2,157).
 void deal(std::vector<Run> runs, int G, Deal& out) {
   if (G > 1)
     std::stable_sort(runs.begin(), runs.end(), [](const Run& a, const Run& b) { return a.cost > b.cost; });
