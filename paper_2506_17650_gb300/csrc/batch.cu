@@ -47,6 +47,7 @@ struct MemberView {
 };
 int member_view(lp_problem* p, MemberView* out);                 // api.cu
 int member_after_batch(lp_problem* p, const DevState& s);         // api.cu
+int member_solve(lp_problem* p, double tol, int64_t iter_limit);  // api.cu
 void set_thread_error(const std::string& msg);                    // api.cu
 
 namespace {
@@ -218,6 +219,7 @@ __device__ __noinline__ void team_promote(const Dev& d, const DevState& s, int r
 // phase and let an FP64 termination test of the promoted point decide.
 __device__ __noinline__ void team_certify(const Dev& d, const Params& prm, DevState& s, int rank, int T, bool wide, double* blk,
                              double (*slots)[kSlots]) {
+  __syncthreads();  // (every warp has read the status that led here)
   if (cta_first()) {
     s.status = 0;
     s.phase32 = 0;
@@ -287,6 +289,7 @@ __device__ bool team_round(const Member& mb, DevState& s, int& budget, int rank,
       if (s.status != 0) break;
       if (sizeof(V) == sizeof(float) && s.phase32) {
         // mixed precision hand-over: at refine_tol, or after refine_stall checks without a 10% gain
+        __syncthreads();  // (every warp has read phase32)
         if (cta_first()) {
           const double kkt = fmax(s.rel_pres, fmax(s.rel_dres, s.rel_gap));
           if (kkt < 0.9 * s.best_kkt) {
@@ -732,7 +735,7 @@ int lp_batch_solve(lp_batch* b, double rel_kkt_tol, int64_t iter_limit, int32_t 
         i = queue.front();
         queue.pop_front();
       }
-      worker_rc[i] = lp_solve(b->probs[i], rel_kkt_tol, iter_limit, nullptr);
+      worker_rc[i] = member_solve(b->probs[i], rel_kkt_tol, iter_limit);
     }
   };
   int rc = LP_OK;
