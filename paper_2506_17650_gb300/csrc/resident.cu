@@ -143,6 +143,34 @@ __device__ __forceinline__ V res_dot(const V* v, const int* c, int count, int mo
   return kChains == 2 ? a[0] + a[kChains - 1] : a[0];
 }
 
+// The same for a row of more than kBlockRowThreshold entries in FP32: pieces of
+// eight terms in FP32, added in FP64, as the step kernels sum such a row.  Only
+// one CTA has such a row in one piece (several cut it into segments); a lane has
+// up to 110 terms of it.  One FP32 chain of 94 equal terms was off by up to 22 x
+// 2^-24 of their sum, the pieces are by less than 2 x 2^-24.  (60 x 4,000 with a
+// row of 4,000 entries, 256 attempts in the FP32 phase: 2,320 us with either.)
+template <int kKind>
+__device__ __noinline__ double res_dot_pieces(const float* v, const int* c, int count, int most,
+                                              const ResGather<float, kKind>& g) {
+  double a = 0.0;
+#pragma unroll 1
+  for (int k0 = 0; k0 < most; k0 += 8) {
+    float p = 0.f;
+#pragma unroll
+    for (int h = 0; h < 8; h += 4) {
+      float xv[4];
+      g.four(c, 32, count - k0 - h, xv);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + h + u < count) p = fma(v[32 * u], xv[u], p);
+      v += 4 * 32;
+      c += 4 * 32;
+    }
+    a += (double)p;
+  }
+  return a;
+}
+
 // The kernel's loop over the attempts is straight-line code that each warp
 // runs once per attempt, so its instruction fetches are on the critical path
 // like every other latency: the pieces below are short loops rather than
@@ -431,6 +459,13 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
         off = e.x + l;
         count = has ? (max(e.y - l, 0) + step - 1) >> lg : 0;
         most = __reduce_max_sync(0xffffffffu, count);
+      }
+      if constexpr (kSolo && sizeof(V) == 4) {
+        if (most > kBlockRowThreshold / 32) {  // (kind 32; a slice's or narrower group's lanes have fewer entries)
+          const double w = lane_sum(res_dot_pieces<kKind>(sv + off, sc + off, count, most, g));
+          if (lane == 0) sum[I.vec] = (V)w;
+          continue;
+        }
       }
       V s;
       if (kBars && far) s = res_dot(far->v + off, far->ci + off, count, most, step, g, &ok);
