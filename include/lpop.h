@@ -185,7 +185,11 @@ int lp_create(int32_t m, int32_t n, int64_t nnz,
  * cumulative, so a second call continues), or until options.time_limit.
  * A check runs before the first attempt and after every check_every-th
  * attempt.  *status_out (may be NULL) receives an lp_status.
- * Errors: LP_ERR_INVALID_ARG (NULL handle, tol < 0), LP_ERR_CUDA.
+ * Errors: LP_ERR_INVALID_ARG (NULL handle, tol < 0), LP_ERR_CUDA.  Where the
+ * call gave up in the middle of an attempt (a wait between its thread blocks
+ * ran out), the iterate is lost: until lp_reset or lp_set_state, lp_solve,
+ * lp_result, lp_get_iterate, lp_get_state and a batch round with this problem
+ * return LP_ERR_CUDA.
  */
 int lp_solve(lp_problem* p, double rel_kkt_tol, int64_t iter_limit, int32_t* status_out);
 

@@ -98,6 +98,9 @@ struct lp_problem {
     bool ok = false;
     ResPlan plan{};
   } res[2];
+  // a resident period gave up in the middle of an attempt: its CTAs stopped at different points of the
+  // update, so that nothing but a new state (lp_reset, lp_set_state) makes sense
+  bool torn = false;
   int* sell_ci[2] = {nullptr, nullptr};
   double* sell_v[2] = {nullptr, nullptr};
   float* sell_v32[2] = {nullptr, nullptr};
@@ -236,6 +239,11 @@ int read_status(lp_problem* p, int* status, int* fault = nullptr) {
   return LP_OK;
 }
 
+int intact(lp_problem* p) {
+  if (!p->torn) return LP_OK;
+  return set_err(p, LP_ERR_CUDA, "the iteration's state was lost when a solve gave up; lp_reset or lp_set_state first");
+}
+
 int init_state(lp_problem* p) {
   DevState s0;
   std::memset(&s0, 0, sizeof(s0));
@@ -256,6 +264,7 @@ int init_state(lp_problem* p) {
   p->best_kkt = INFINITY;
   p->stall = 0;
   CK(cudaStreamSynchronize(p->stream));
+  p->torn = false;
   p->initial_check_done = false;
   p->solved_once = false;
   p->host_attempts = 0;
@@ -694,6 +703,7 @@ int upload_vec(lp_problem* p, double* ddst, const double* host, int len, const i
 }
 
 int get_state_impl(lp_problem* p, double* vn, double* vm, double* scal) {
+  TRY(intact(p));
   TRY(select_device(p));
   launch_flush_update(p->d, p->prm, p->fp32_phase, p->stream);
   CK(cudaGetLastError());
@@ -768,6 +778,7 @@ int set_state_impl(lp_problem* p, const double* vn, const double* vm, const doub
   if (p->fp32_phase) launch_demote_state(p->d, p->stream);  // the FP32 phase continues from the imported state
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(p->stream));
+  p->torn = false;
   p->host_attempts = hs.attempts;
   p->initial_check_done = scal[14] != 0.0;
   p->solved_once = false;
@@ -1020,6 +1031,7 @@ const ResPlan* resident_plan(lp_problem* p, int* rc) {
     h.plan.seg = h.plan.ctl + h.plan.G + 8;
     h.plan.gx = R.block + o3;
     h.plan.bar = reinterpret_cast<unsigned int*>(R.block + o4);
+    h.plan.test = R.plan.test;
     R.plan = h.plan;
     R.ok = true;
     return LP_OK;
@@ -1029,6 +1041,7 @@ const ResPlan* resident_plan(lp_problem* p, int* rc) {
 }
 
 int solve_impl(lp_problem* p, double tol, int64_t iter_limit, int32_t* status_out, bool resident = true) {
+  TRY(intact(p));
   TRY(select_device(p));
   const auto t0 = std::chrono::steady_clock::now();
   const int ce = p->opt.check_every;
@@ -1069,7 +1082,10 @@ int solve_impl(lp_problem* p, double tol, int64_t iter_limit, int32_t* status_ou
       if (fault) {
         CK(cudaMemsetAsync(&p->d.st->fault, 0, sizeof(int), p->stream));
         p->res[fp32 ? 1 : 0].ok = false;  // the two-kernel path from here on
-        if (fault == 1) return set_err(p, LP_ERR_CUDA, "a resident check period gave up waiting for its CTAs");
+        if (fault == 1) {
+          p->torn = true;
+          return set_err(p, LP_ERR_CUDA, "a resident check period gave up waiting for its CTAs");
+        }
         continue;  // nothing ran
       }
       p->launches += 1 + (checked ? check_kernel_count() : 0);
@@ -1163,6 +1179,9 @@ int member_solve(lp_problem* p, double tol, int64_t iter_limit) {
   }
 }
 
+// Whether a problem has a state to go on from.
+int member_intact(lp_problem* p) { return p ? intact(p) : LP_ERR_INVALID_ARG; }
+
 // Host-side view of a problem after a batched kernel advanced its device state.
 int member_after_batch(lp_problem* p, const DevState& s) {
   if (!p) return LP_ERR_INVALID_ARG;
@@ -1235,6 +1254,7 @@ int lp_solve(lp_problem* p, double rel_kkt_tol, int64_t iter_limit, int32_t* sta
 int lp_result(lp_problem* p, double* x, double* y, lp_stats* st) {
   if (!p) return set_err(nullptr, LP_ERR_INVALID_ARG, "problem handle is NULL");
   if (!p->solved_once) return set_err(p, LP_ERR_NOT_SOLVED, "lp_result called before lp_solve");
+  TRY(intact(p));
   TRY(select_device(p));
   DevState hs;
   const int n = p->d.n, m = p->d.m;
@@ -1265,6 +1285,7 @@ int lp_result(lp_problem* p, double* x, double* y, lp_stats* st) {
 
 int lp_get_iterate(lp_problem* p, double* x, double* y, double* T, double* Sigma, double* scal) {
   if (!p) return set_err(nullptr, LP_ERR_INVALID_ARG, "problem handle is NULL");
+  TRY(intact(p));
   TRY(select_device(p));
   launch_flush_update(p->d, p->prm, p->fp32_phase, p->stream);
   CK(cudaGetLastError());
@@ -1384,6 +1405,19 @@ int lpop_bad_gathers(lp_problem* p, unsigned long long* count) {
   unsigned int h = 0;
   if (cudaMemcpy(&h, p->d.bad_gathers, sizeof(h), cudaMemcpyDeviceToHost) != cudaSuccess) return LP_ERR_CUDA;
   *count = h;
+  return LP_OK;
+}
+
+// Checked builds only: limits of the waits of the problem's resident periods (0: the usual ones), and
+// arrivals at their start and numbers of words within an attempt that never come.
+int lpop_resident_limits(lp_problem* p, int start_spins, int spins, int missing_arrivals, int missing_words) {
+  if (!p) return LP_ERR_INVALID_ARG;
+  for (lp_problem::Resident& R : p->res) {
+    R.plan.test.start_spins = start_spins;
+    R.plan.test.spins = spins;
+    R.plan.test.missing_arrivals = missing_arrivals;
+    R.plan.test.missing_words = missing_words;
+  }
   return LP_OK;
 }
 #endif

@@ -47,6 +47,7 @@ struct MemberView {
 };
 int member_view(lp_problem* p, MemberView* out);                 // api.cu
 int member_after_batch(lp_problem* p, const DevState& s);         // api.cu
+int member_intact(lp_problem* p);                                 // api.cu
 int member_solve(lp_problem* p, double tol, int64_t iter_limit);  // api.cu
 void set_thread_error(const std::string& msg);                    // api.cu
 
@@ -669,6 +670,9 @@ int lp_batch_round(lp_batch* b, double rel_kkt_tol, int32_t attempts, int64_t it
     if (active_out) *active_out = 0;
     return LP_OK;
   }
+  for (int i = 0; i < count; ++i)
+    if ((b->handed.empty() || !b->handed[i]) && member_intact(b->probs[i]) != LP_OK)
+      return berr(b, LP_ERR_CUDA, "member " + std::to_string(i) + " lost its state in a solve; reset it first");
   int rc = read_states(b);
   if (rc != LP_OK) return rc;
   // members still running, and members that stopped under another tolerance

@@ -33,6 +33,20 @@ namespace {
 constexpr int kStartSpins = 1 << 21;  // polls (~0.3 us each) before a launch gives up on its CTAs all being there
 constexpr int kSpins = 1 << 23;       // ... and before a wait for another CTA's word gives up
 
+// The checked build takes both limits from the plan, with an arrival or a word
+// that never comes, so that a test can let a wait run out.
+#ifdef LPOP_CHECK_BOUNDS
+__device__ __forceinline__ int start_spins(const ResPlan& pl) { return pl.test.start_spins ? pl.test.start_spins : kStartSpins; }
+__device__ __forceinline__ int wait_spins(const ResPlan& pl) { return pl.test.spins ? pl.test.spins : kSpins; }
+__device__ __forceinline__ unsigned int missing_arrivals(const ResPlan& pl) { return (unsigned int)pl.test.missing_arrivals; }
+__device__ __forceinline__ unsigned int missing_words(const ResPlan& pl) { return (unsigned int)pl.test.missing_words; }
+#else
+__device__ __forceinline__ constexpr int start_spins(const ResPlan&) { return kStartSpins; }
+__device__ __forceinline__ constexpr int wait_spins(const ResPlan&) { return kSpins; }
+__device__ __forceinline__ constexpr unsigned int missing_arrivals(const ResPlan&) { return 0u; }
+__device__ __forceinline__ constexpr unsigned int missing_words(const ResPlan&) { return 0u; }
+#endif
+
 // The word of one element of x+ or y+.
 template <class V>
 struct ResElt;
@@ -83,6 +97,7 @@ struct ResGather {
   unsigned int seq;
   int n;
   unsigned int* bad;
+  int spins;
   // xv[u] = x[c[u step]] for u < min(4, count); false if a word did not come
   __device__ __forceinline__ bool four(const int* c, int step, int count, V (&xv)[4]) const {
     const int none = -1;
@@ -104,7 +119,7 @@ struct ResGather {
         if (j[u] != none) xv[u] = x[j[u]];
       return true;
     } else {
-      for (int t = 0; t < kSpins; ++t) {
+      for (int t = 0; t < spins; ++t) {
         bool here = true;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -147,8 +162,8 @@ __device__ __forceinline__ V res_dot(const V* v, const int* c, int count, int mo
 // eight terms in FP32, added in FP64, as the step kernels sum such a row.  Only
 // one CTA has such a row in one piece (several cut it into segments); a lane has
 // up to 110 terms of it.  One FP32 chain of 94 equal terms was off by up to 22 x
-// 2^-24 of their sum, the pieces are by less than 2 x 2^-24.  (60 x 4,000 with a
-// row of 4,000 entries, 256 attempts in the FP32 phase: 2,320 us with either.)
+// 2^-24 of their sum, the pieces are by less than 2 x 2^-24.  (4 x 2,500 with a
+// full row, 256 attempts in the FP32 phase: 2,122 us with the chain, 1,986 so.)
 template <int kKind>
 __device__ __noinline__ double res_dot_pieces(const float* v, const int* c, int count, int most,
                                               const ResGather<float, kKind>& g) {
@@ -208,12 +223,12 @@ __device__ __forceinline__ bool bar_wait(const unsigned int* bar, unsigned int t
 
 // Sum over the CTAs of one field's records of this attempt (all lanes of the
 // calling warp); false when they did not all come.
-__device__ __forceinline__ bool rec_sum(const ulonglong2* rec, int G, unsigned int seq, double* out) {
+__device__ __forceinline__ bool rec_sum(const ulonglong2* rec, int G, unsigned int seq, int spins, double* out) {
   const int lane = threadIdx.x & 31;
   constexpr int K = kResMaxCtas / 32;
   double v[K];
   bool done = false;
-  for (int k = 0; k < kSpins && !done; ++k) {
+  for (int k = 0; k < spins && !done; ++k) {
     bool mine = true;
 #pragma unroll
     for (int q = 0; q < K; ++q) {
@@ -415,7 +430,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
     __syncthreads();
     if (tid == 0) {
       bar_arrive(pl.bar);
-      const bool all = bar_wait(pl.bar, arrived + pl.G, kStartSpins);
+      const bool all = bar_wait(pl.bar, arrived + pl.G + missing_arrivals(pl), start_spins(pl));
       const unsigned int was = atomicCAS(pl.bar + 2, 0u, all ? 1u : 2u);
       s_ok = was == 0u ? all : was == 1u;
       if (!s_ok) d.st->fault = 2;
@@ -436,8 +451,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
     for (int i = warp - w0; i < n; i += kResWarps - w0) {
       const ResItem& I = it[i];
       if (!kSolo && I.kind == kOwnKind) {  // the segments' sums, in segment order over the lanes
-        double t;
-        ok = rec_sum(pl.seg + I.ent, I.len, g.seq, &t) && ok;
+        double t = 0.0;
+        ok = ok && rec_sum(pl.seg + I.ent, I.len, g.seq, g.spins, &t);
         if (lane == 0) sum[I.vec] = (V)t;
         continue;
       }
@@ -539,7 +554,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
         target += pl.G;
         if (tid == 0) {
           bar_arrive(pl.bar);
-          if (!bar_wait(pl.bar, target, kSpins)) s_ok = 0;
+          if (!bar_wait(pl.bar, target + missing_words(pl), wait_spins(pl))) s_ok = 0;
         }
         __syncthreads();
         if (!s_ok) {
@@ -552,7 +567,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
       V* const axc = dax + cur * pl.rd;
       V* const axn = dax + nxt * pl.rd;
       row_sums(s_it + np, nd, s_vd, s_cd, s_lrp + C.nlp, s_lend, pl.far & 2 ? &far_a : nullptr,
-               ResGather<V, kKind>{kSolo ? xn : v.x[nxt], gxw, seq, d.n, d.bad_gathers}, axn, 0);
+               ResGather<V, kKind>{kSolo ? xn : v.x[nxt], gxw, seq + missing_words(pl), d.n, d.bad_gathers, wait_spins(pl)}, axn, 0);
       __syncthreads();
       V accd[4] = {V(0), V(0), V(0), V(0)};
 #pragma unroll 1
@@ -623,7 +638,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
             if (blockIdx.x == 0) {
               __syncwarp();
               double t;
-              ok = rec_sum(pl.rec + f * pl.G, pl.G, seq, &t) && ok;
+              ok = rec_sum(pl.rec + f * pl.G, pl.G, seq, wait_spins(pl), &t) && ok;
               if (lane == 0) s_tot[f] = t;
             }
           }
@@ -647,7 +662,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
         } else if (warp == 0) {
           double w = 0.0;
           bool here = false;
-          for (int k = 0; k < kSpins && !here; ++k)
+          for (int k = 0; k < wait_spins(pl) && !here; ++k)
             here = __all_sync(0xffffffffu, lane >= 8 || ResElt<double>::get(pl.ctl + (blockIdx.x & ~7u) + lane, seq, &w));
           if (!here) s_ok = 0;
           if (lane < 8) bcast_read(s_st, lane, w);
@@ -658,12 +673,13 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
       if (kBars && a >= 0) {
         if (tid == 32 * kCtlWarps) {
           bar_arrive(pl.bar);
-          if (!bar_wait(pl.bar, target + pl.G, kSpins)) s_ok = 0;
+          if (!bar_wait(pl.bar, target + pl.G, wait_spins(pl))) s_ok = 0;
         }
         rows_sync();
       }
       row_sums(s_it, np, s_vp, s_cp, s_lrp, s_lenp, pl.far & 1 ? &far_at : nullptr,
-               ResGather<V, kKind>{kSolo ? yn : v.y[nxt], gyw + (size_t)nxt * d.m, seq, d.m, d.bad_gathers}, psum + nxt * pl.rp, kCtlWarps);
+               ResGather<V, kKind>{kSolo ? yn : v.y[nxt], gyw + (size_t)nxt * d.m, seq, d.m, d.bad_gathers, wait_spins(pl)}, psum + nxt * pl.rp,
+               kCtlWarps);
       if (avg) {  // the last accepted attempt's terms of the averages
         const int t0 = tid - 32 * kCtlWarps, step = kResThreads - 32 * kCtlWarps;
 #pragma unroll 1

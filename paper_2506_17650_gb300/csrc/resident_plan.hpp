@@ -62,6 +62,11 @@ struct ResPlan {
   int segs, segs_d;                // segments of both sides, and of A
   int longest;                     // entries of the longest row of A or A^T
   int smem;                        // dynamic shared memory, bytes
+  // read by the checked build only: shorter limits of the waits (0: the usual ones), arrivals at the start and
+  // numbers of words (or arrivals) within an attempt that nothing reaches
+  struct {
+    int start_spins, spins, missing_arrivals, missing_words;
+  } test;
 };
 
 // Byte offsets of a CTA's arrays in dynamic shared memory.

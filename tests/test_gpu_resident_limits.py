@@ -1,0 +1,84 @@
+"""Resident check periods whose waits run out.
+
+In the checked build the limits of the waits can be made short, and an arrival
+or a word can be awaited that nothing ever sends (lpop_resident_limits): the
+kernel gives up after the limit, sets its error status and returns.  Nothing
+faults or hangs.
+"""
+import subprocess
+import sys
+
+import pytest
+
+from paper_2506_17650_gb300 import build as lpbuild
+from tests.conftest import ROOT
+
+pytestmark = pytest.mark.gpu
+
+PRELUDE = r'''
+import ctypes, sys
+import numpy as np
+root, lib, case = sys.argv[1:4]
+sys.path.insert(0, root)
+import lpgen
+import paper_2506_17650_gb300 as lpop
+lpop.load_library(lib)
+raw = ctypes.CDLL(lib)
+lps = {
+    "words": lambda: lpgen.batch_member(9, 701, 1_753),
+    "barriers": lambda: lpgen.row_length_mix(2),
+    "far": lambda: lpgen.powerlaw(2, 50_000, 125_000, 800_000),
+}
+KEYS = ("x", "y", "T", "Sigma", "ax", "xbar", "ybar", "GT", "GS")
+
+
+def limits(p, **k):
+    args = [k.get(n, 0) for n in ("start_spins", "spins", "missing_arrivals", "missing_words")]
+    assert raw.lpop_resident_limits(p.handle, *args) == 0
+
+
+def error(fn):
+    try:
+        fn()
+    except lpop.LpError as e:
+        return e.code
+    return None
+
+
+lp = lps[case]()
+p = lpop.Problem(lp, alpha=1e-4, phi=7)
+'''
+
+
+def _run(script, case):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    lib = lpbuild.build(checked=True)
+    subprocess.run([sys.executable, "-c", PRELUDE + script, ROOT, lib, case], check=True, timeout=600)
+
+
+LOST = r'''
+p.solve(0.0, 64)
+start = p.get_state()
+limits(p, spins=500, missing_words=1)
+assert error(lambda: p.solve(0.0, 128)) == lpop.LP_ERR_CUDA
+limits(p)
+with lpop.Batch([p]) as b:
+    for call in (lambda: p.solve(0.0, 192), p.result, p.get_state, p.iterate, lambda: b.round(0.0, 64, 192)):
+        assert error(call) == lpop.LP_ERR_CUDA, call
+p.set_state(start)
+again = p.get_state()
+assert all(np.array_equal(again[k], start[k]) for k in KEYS)
+p.solve(0.0, 128)
+assert p.get_state()["attempts"] == 128
+p.reset()
+p.solve(0.0, 64)
+x, y, st = p.result()
+assert st["iterations"] == 64 and np.all(np.isfinite(x)) and np.all(np.isfinite(y))
+'''
+
+
+@pytest.mark.parametrize("case", ["words", "barriers", "far"])
+def test_state_lost_in_a_period_is_refused_until_it_is_set_again(case):
+    _run(LOST, case)
