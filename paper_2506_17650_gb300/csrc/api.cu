@@ -96,7 +96,9 @@ struct lp_problem {
     char* block = nullptr;
     bool tried = false;
     bool ok = false;
+    bool alone = true;  // the launch may be resident (false once one was refused or not all of its CTAs started)
     ResPlan plan{};
+    cudaGraphExec_t gexec = nullptr;  // a check period of the plan's stepped launches
   } res[2];
   // a resident period gave up in the middle of an attempt: its CTAs stopped at different points of the
   // update, so that nothing but a new state (lp_reset, lp_set_state) makes sense
@@ -629,13 +631,18 @@ int create_events(lp_problem* p) {
 
 bool sampled(const lp_problem* p, int a) { return p->opt.kernel_timing && (a % timing_stride(p)) == 0; }
 
-int capture_graph(lp_problem* p, bool fp32) {
-  cudaGraphExec_t* slot = fp32 ? &p->gexec32 : &p->gexec;
+// One check period as a graph: of the two step kernels or, with a plan, of its stepped launches.
+int capture_graph(lp_problem* p, bool fp32, const ResPlan* plan = nullptr) {
+  cudaGraphExec_t* slot = plan ? &p->res[fp32 ? 1 : 0].gexec : fp32 ? &p->gexec32 : &p->gexec;
   if (*slot) return LP_OK;
   cudaGraph_t g = nullptr;
   CK(cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal));
   const int ce = p->opt.check_every;
   for (int a = 0; a < ce; ++a) {
+    if (plan) {
+      launch_stepped(p->d, p->prm, *plan, fp32, p->stream);
+      continue;
+    }
     const bool tm = sampled(p, a);
     const int sidx = a / (p->opt.kernel_timing ? timing_stride(p) : 1);
     if (tm) cudaEventRecordWithFlags(p->events[3 * sidx], p->stream, cudaEventRecordExternal);
@@ -791,6 +798,8 @@ void release(lp_problem* p) {
   if (p->stream) cudaStreamSynchronize(p->stream);
   if (p->gexec) cudaGraphExecDestroy(p->gexec);
   if (p->gexec32) cudaGraphExecDestroy(p->gexec32);
+  for (lp_problem::Resident& R : p->res)
+    if (R.gexec) cudaGraphExecDestroy(R.gexec);
   for (auto e : p->events)
     if (e) cudaEventDestroy(e);
   for (void* v : p->allocs) cudaFree(v);
@@ -1004,7 +1013,10 @@ const ResPlan* resident_plan(lp_problem* p, int* rc) {
   auto build = [&]() -> int {
     const int esize = p->fp32_phase ? 4 : 8;
     int limit = 0;
-    CK(resident_smem_limit(p->device, &limit));
+    if (resident_smem_limit(p->device, &limit) != cudaSuccess) {
+      cudaGetLastError();
+      return LP_OK;
+    }
     std::vector<int> head[2];
     for (int which = 0; which < 2; ++which) {
       head[which].assign((size_t)resident_long_rows(which ? p->d.binsAt : p->d.binsA) + 1, 0);
@@ -1040,6 +1052,55 @@ const ResPlan* resident_plan(lp_problem* p, int* rc) {
   return R.ok ? &R.plan : nullptr;
 }
 
+// A (part of a) check period in one launch.  *ran: false, with nothing done,
+// where the launch was refused (a context that may use part of the SMs) or not
+// all of its CTAs started within the limit: then the plan's stepped launches
+// take over for good, with the same bits (with one CTA: the two step kernels).
+int run_resident(lp_problem* p, const ResPlan& plan, bool fp32, int nrun, bool check, bool* ran, int* status) {
+  lp_problem::Resident& R = p->res[fp32 ? 1 : 0];
+  *ran = false;
+  if (!R.alone) return LP_OK;
+  int fault = 0;
+  {
+    SmLease lease(p->device, p->sms, plan.G > 1 ? plan.G : 0, plan.G);
+    if (launch_resident(p->d, p->prm, plan, fp32, nrun, p->stream) != cudaSuccess) {
+      cudaGetLastError();
+      R.alone = false;
+      R.ok = plan.G > 1;
+      return LP_OK;
+    }
+    if (check) launch_check(p->d, p->prm, 0, fp32, p->stream);
+    CK(cudaGetLastError());
+    TRY(read_status(p, status, &fault));
+  }
+  if (fault) {
+    CK(cudaMemsetAsync(&p->d.st->fault, 0, sizeof(int), p->stream));
+    R.alone = false;
+    if (fault == 1) {
+      p->torn = true;
+      return set_err(p, LP_ERR_CUDA, "a resident check period gave up waiting for its CTAs");
+    }
+    return LP_OK;
+  }
+  p->launches += 1 + (check ? check_kernel_count() : 0);
+  *ran = true;
+  return LP_OK;
+}
+
+// The same in two launches per attempt.
+int run_stepped(lp_problem* p, const ResPlan& plan, bool fp32, int nrun, bool check, int* status) {
+  if (p->opt.use_graph && nrun == p->opt.check_every) {
+    TRY(capture_graph(p, fp32, &plan));
+    CK(cudaGraphLaunch(p->res[fp32 ? 1 : 0].gexec, p->stream));
+  } else {
+    for (int a = 0; a < nrun; ++a) launch_stepped(p->d, p->prm, plan, fp32, p->stream);
+    if (check) launch_check(p->d, p->prm, 0, fp32, p->stream);
+    CK(cudaGetLastError());
+  }
+  p->launches += 2LL * nrun + (check ? check_kernel_count() : 0);
+  return read_status(p, status);
+}
+
 int solve_impl(lp_problem* p, double tol, int64_t iter_limit, int32_t* status_out, bool resident = true) {
   TRY(intact(p));
   TRY(select_device(p));
@@ -1071,24 +1132,10 @@ int solve_impl(lp_problem* p, double tol, int64_t iter_limit, int32_t* status_ou
     if (plan) {
       const long long nrun = to_boundary < remaining ? to_boundary : remaining;
       checked = nrun == to_boundary;
-      int fault = 0;
-      {
-        SmLease lease(p->device, p->sms, plan->G > 1 ? plan->G : 0, plan->G);
-        CK(launch_resident(p->d, p->prm, *plan, fp32, (int)nrun, p->stream));
-        if (checked) launch_check(p->d, p->prm, 0, fp32, p->stream);
-        CK(cudaGetLastError());
-        TRY(read_status(p, &status, &fault));
-      }
-      if (fault) {
-        CK(cudaMemsetAsync(&p->d.st->fault, 0, sizeof(int), p->stream));
-        p->res[fp32 ? 1 : 0].ok = false;  // the two-kernel path from here on
-        if (fault == 1) {
-          p->torn = true;
-          return set_err(p, LP_ERR_CUDA, "a resident check period gave up waiting for its CTAs");
-        }
-        continue;  // nothing ran
-      }
-      p->launches += 1 + (checked ? check_kernel_count() : 0);
+      bool ran = false;
+      TRY(run_resident(p, *plan, fp32, (int)nrun, checked, &ran, &status));
+      if (!ran && !p->res[fp32 ? 1 : 0].ok) continue;  // (the two step kernels from here on)
+      if (!ran) TRY(run_stepped(p, *plan, fp32, (int)nrun, checked, &status));
       p->host_attempts += nrun;
     } else if (p->opt.use_graph && to_boundary == ce && remaining >= ce) {
       TRY(capture_graph(p, fp32));
@@ -1409,14 +1456,15 @@ int lpop_bad_gathers(lp_problem* p, unsigned long long* count) {
 }
 
 // Checked builds only: limits of the waits of the problem's resident periods (0: the usual ones), and
-// arrivals at their start and numbers of words within an attempt that never come.
-int lpop_resident_limits(lp_problem* p, int start_spins, int spins, int missing_arrivals, int missing_words) {
+// arrivals at their start and numbers of words within an attempt that never come, or launches refused.
+int lpop_resident_limits(lp_problem* p, int start_spins, int spins, int missing_arrivals, int missing_words, int refuse) {
   if (!p) return LP_ERR_INVALID_ARG;
   for (lp_problem::Resident& R : p->res) {
     R.plan.test.start_spins = start_spins;
     R.plan.test.spins = spins;
     R.plan.test.missing_arrivals = missing_arrivals;
     R.plan.test.missing_words = missing_words;
+    R.plan.test.refuse = refuse;
   }
   return LP_OK;
 }

@@ -243,6 +243,18 @@ __device__ __forceinline__ bool rec_sum(const ulonglong2* rec, int G, unsigned i
   return done;
 }
 
+// The same sum over words that are known to be there.
+__device__ __forceinline__ double sum_words(const ulonglong2* rec, int G) {
+  const int lane = threadIdx.x & 31;
+  double v[kResMaxCtas / 32];
+#pragma unroll
+  for (int q = 0; q < kResMaxCtas / 32; ++q) {
+    const int g = lane + 32 * q;
+    v[q] = g < G ? __longlong_as_double((long long)__ldcg(&rec[g].x)) : 0.0;
+  }
+  return lane_sum(((v[0] + v[1]) + (v[2] + v[3])) + v[4]);
+}
+
 constexpr int kFacs = 64;
 constexpr int kCtlWarps = 3;  // warps that sum the records (a field each); warp 0 then runs the step control
 
@@ -729,6 +741,158 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
   }
 }
 
+// ---- the same attempts in two plain launches each --------------------------------
+//
+// A stepped period does what a resident one does, row for row and sum for sum in
+// the same order, so that the two give the same bits, but its blocks wait for
+// nothing: the plan's CTAs are the blocks of two launches per attempt (A^T y and
+// x+; A x+, y+ and, in the last block to finish, the step control), which read
+// the matrix and the vectors from global memory (L2).  It is what a period runs as when
+// the SMs for a resident one are not to be had.
+//
+// Sums of long rows (several segments): the block that has the row forms all of them.
+template <class V, bool kPrimal>
+__global__ void __launch_bounds__(kResThreads, 2) stepped_kernel(Dev d, Params prm, ResPlan pl) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  __shared__ double s_red[4 * kResThreads];
+  __shared__ double s_tot[8];
+  __shared__ double s_fac[2];
+  __shared__ DevState s_st;
+  __shared__ int s_last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();
+  const ResCta C = pl.cta[blockIdx.x];
+  const ResItem* const it = pl.items + (kPrimal ? C.p0 : C.d0);
+  const int items = kPrimal ? C.p1 - C.p0 : C.d1 - C.d0, rows = kPrimal ? C.rp : C.rd;
+  V* const s_sum = reinterpret_cast<V*>(s_raw);  // by local row
+  int* const s_row = reinterpret_cast<int*>(s_sum + (kPrimal ? pl.rp : pl.rd));
+  const Vecs<V>& v = vecs<V>(d);
+  const CsrT<V> M = kPrimal ? csr_at<V>(d) : csr_a<V>(d);
+  std::conditional_t<kPrimal, PrimalOp<V, true>, DualOp<V, true>> op;
+  op.sc = read_scalars<V>(d.st, kPrimal);
+  const int cur = op.sc.cur;
+  if constexpr (kPrimal) op.bind(v, prm, cur);
+  else op.bind(v, prm, d.sense, cur);
+  const bool collect = op.sc.collect != 0;
+  const ResGather<V, kBarriersKind> g{kPrimal ? v.y[cur] : v.x[cur ^ 1], nullptr, 0u, kPrimal ? d.m : d.n, d.bad_gathers, 0};
+  bool ok = true;
+  // ---- row sums -----------------------------------------------------------------
+  int own = items;  // the rows cut into segments come last
+  while (own > 0 && it[own - 1].kind == kOwnKind) --own;
+#pragma unroll 1
+  for (int i = warp; i < own; i += kResWarps) {
+    const ResItem I = it[i];
+    if (I.kind == kSegKind) continue;
+    if (lane < I.nrows) s_row[I.vec + lane] = I.row0 + lane;
+    const int width = I.kind == 0 ? 1 : I.kind, lg = 31 - __clz(width);
+    const int l = lane & (width - 1), r = lane >> lg;
+    const bool has = r < I.nrows;
+    const int e0 = has ? M.rp[I.row0 + r] : 0, len = has ? M.rp[I.row0 + r + 1] - e0 : 0;
+    const int count = max(len - l + width - 1, 0) >> lg;
+    const int most = __reduce_max_sync(0xffffffffu, count);
+    V s = res_dot(M.v + e0 + l, M.ci + e0 + l, count, most, width, g, &ok);
+#pragma unroll 1
+    for (int o = width / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, width);
+    if (l == 0 && has) s_sum[I.vec + r] = s;
+  }
+  if (own < items) {
+    int at = 0;  // segments of the rows before
+#pragma unroll 1
+    for (int i = own; i < items; ++i) {
+      const ResItem I = it[i];
+      const int e0 = M.rp[I.row0], e1 = M.rp[I.row0 + 1];
+#pragma unroll 1
+      for (int k = (warp - at) & (kResWarps - 1); k < I.len; k += kResWarps) {
+        const int beg = e0 + k * kResSeg, size = min(kResSeg, e1 - beg);
+        const V s = res_dot(M.v + beg + lane, M.ci + beg + lane, (size - lane + 31) >> 5, (size + 31) >> 5, 32, g, &ok);
+        const double w = lane_sum((double)s);
+        if (lane == 0) pl.seg[I.ent + k].x = (unsigned long long)__double_as_longlong(w);
+      }
+      at += I.len;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = own + warp; i < items; i += kResWarps) {
+      const ResItem I = it[i];
+      const double t = sum_words(pl.seg + I.ent, I.len);
+      if (lane == 0) {
+        s_sum[I.vec] = (V)t;
+        s_row[I.vec] = I.row0;
+      }
+    }
+  }
+  __syncthreads();
+  // ---- x+ or y+ -------------------------------------------------------------------
+#pragma unroll 1
+  for (int t = tid; t < rows; t += kResThreads) {
+    const V s[1] = {s_sum[t]};
+    op.prefetch(s_row[t]);
+    op.row(s_row[t], s);
+  }
+  // ---- this block's record ----------------------------------------------------------
+  constexpr int kAcc = kPrimal ? 3 : 4;
+#pragma unroll
+  for (int q = 0; q < kAcc; ++q) s_red[q * kResThreads + tid] = (double)op.acc[q];
+  __syncthreads();
+  const int field[2][4] = {{0, 1, 3, 4}, {2, 5, 6, 0}};  // (as in resident_kernel: the last four only where they are recorded)
+  if (warp < (collect ? kAcc : kPrimal ? 1 : 2)) {
+    const double t = res_sum(s_red + warp * kResThreads, min(kResWarps, (rows + 31) / 32));
+    if (lane == 0) s_tot[warp] = t;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int q = 0; q < (collect ? kAcc : kPrimal ? 1 : 2); ++q)
+      pl.rec[field[kPrimal][q] * pl.G + blockIdx.x].x = (unsigned long long)__double_as_longlong(s_tot[q]);
+    if (!kPrimal) {
+      unsigned int t;
+      asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(t) : "l"(pl.bar + 4) : "memory");
+      s_last = t == gridDim.x - 1;
+    }
+  }
+  if constexpr (kPrimal) {
+    pdl_trigger();
+  } else {
+    __syncthreads();
+    if (!s_last) return;
+    pdl_trigger();
+    // ---- totals and step control ----------------------------------------------------
+    double* const sd = reinterpret_cast<double*>(&s_st);
+    for (int t = tid; t < (int)(sizeof(DevState) / 8); t += kResThreads) sd[t] = reinterpret_cast<const double*>(d.st)[t];
+    if (warp < (collect ? 7 : 3)) {
+      const double t = sum_words(pl.rec + warp * pl.G, pl.G);
+      if (lane == 0) s_tot[warp] = t;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      step_factors(d.step_tab, s_st.attempts + 1, s_fac, s_fac + 1);
+      const double t1[3] = {s_tot[2], collect ? s_tot[5] : 0.0, collect ? s_tot[6] : 0.0};
+      const double t2[4] = {s_tot[0], s_tot[1], collect ? s_tot[3] : 0.0, collect ? s_tot[4] : 0.0};
+      step_control_state(s_st, prm, s_fac[0], s_fac[1], t1, t2);
+      pl.bar[4] = 0u;
+    }
+    __syncthreads();
+    for (int t = tid; t < (int)(sizeof(DevState) / 8); t += kResThreads) reinterpret_cast<double*>(d.st)[t] = sd[t];
+  }
+}
+
+constexpr int kSteppedSmem = 56 * 1024;
+int stepped_smem(const ResPlan& pl, bool fp32) { return (pl.rp > pl.rd ? pl.rp : pl.rd) * ((fp32 ? 4 : 8) + 4); }
+
+template <class V, bool kPrimal>
+void launch_stepped_half(const Dev& d, const Params& prm, const ResPlan& pl, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)pl.G, 1, 1);
+  cfg.blockDim = dim3(kResThreads, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)stepped_smem(pl, sizeof(V) == 4);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, stepped_kernel<V, kPrimal>, d, prm, pl);  // errors surface through cudaGetLastError
+}
+
 template <class V>
 const void* resident_fn_t(int kind) {
   if (kind == kSoloKind) return (const void*)resident_kernel<V, kSoloKind>;
@@ -753,6 +917,8 @@ int resident_kind(const ResPlan& pl) {
 
 }  // namespace
 
+// Dynamic shared memory that a resident CTA may take; also lets the stepped kernels have theirs
+// (at most 5,800 rows of a CTA by 8 bytes, or 3,200 by 12).
 cudaError_t resident_smem_limit(int device, int* bytes) {
   int optin = 0;
   cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
@@ -768,12 +934,20 @@ cudaError_t resident_smem_limit(int device, int* bytes) {
     if (e != cudaSuccess) return e;
     least = std::min(least, room);
   }
+  for (const void* fn : {(const void*)stepped_kernel<double, true>, (const void*)stepped_kernel<double, false>,
+                         (const void*)stepped_kernel<float, true>, (const void*)stepped_kernel<float, false>}) {
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSteppedSmem);
+    if (e != cudaSuccess) return e;
+  }
   *bytes = least;
   return cudaSuccess;
 }
 
 cudaError_t launch_resident(const Dev& d, const Params& prm, const ResPlan& pl, bool fp32, int attempts,
                             cudaStream_t s) {
+#ifdef LPOP_CHECK_BOUNDS
+  if (pl.test.refuse) return cudaErrorCooperativeLaunchTooLarge;
+#endif
   Dev da = d;
   Params pa = prm;
   ResPlan pp = pl;
@@ -781,6 +955,16 @@ cudaError_t launch_resident(const Dev& d, const Params& prm, const ResPlan& pl, 
   const void* fn = resident_fn(fp32, resident_kind(pl));
   if (pl.G == 1) return cudaLaunchKernel(fn, dim3(1), dim3(kResThreads), args, (size_t)pl.smem, s);
   return cudaLaunchCooperativeKernel(fn, dim3((unsigned)pl.G), dim3(kResThreads), args, (size_t)pl.smem, s);
+}
+
+void launch_stepped(const Dev& d, const Params& prm, const ResPlan& pl, bool fp32, cudaStream_t s) {
+  if (fp32) {
+    launch_stepped_half<float, true>(d, prm, pl, s);
+    launch_stepped_half<float, false>(d, prm, pl, s);
+  } else {
+    launch_stepped_half<double, true>(d, prm, pl, s);
+    launch_stepped_half<double, false>(d, prm, pl, s);
+  }
 }
 
 SmTokens& sm_tokens(int device, int sms) {

@@ -24,6 +24,8 @@ namespace lpop {
 // Up to `attempts` step attempts in one launch (cooperative when G > 1).
 cudaError_t launch_resident(const Dev& d, const Params& prm, const ResPlan& pl, bool fp32, int attempts,
                             cudaStream_t s);
+// One step attempt of the plan in two plain launches, with the same bits (G > 1).
+void launch_stepped(const Dev& d, const Params& prm, const ResPlan& pl, bool fp32, cudaStream_t s);
 cudaError_t resident_smem_limit(int device, int* bytes);  // dynamic shared memory a CTA may take
 
 // The SMs of a device (shared by every problem and batch on it).

@@ -55,7 +55,8 @@ struct ResPlan {
   ulonglong2* ctl;    // [8 * (G / 8 + 1)] result of the step control, a line for each eight CTAs
   ulonglong2* seg;    // words of the segments: those of A^T, then those of A
   void* gx;           // words of x+ [n], then of y+ [2][m]
-  unsigned int* bar;  // arrivals, number of the last attempt, start decision, arrivals before this launch
+  unsigned int* bar;  // arrivals, number of the last attempt, start decision, arrivals before this launch; [4]: a
+                      // stepped launch's finished blocks
   int G;
   int ep, ed, rp, rd, lp, ld, it;  // entries, rows, long rows of A^T / A; items of both
   int far;                         // 1: the entries of A^T, 2: those of A are read from the global CSR arrays
@@ -63,9 +64,9 @@ struct ResPlan {
   int longest;                     // entries of the longest row of A or A^T
   int smem;                        // dynamic shared memory, bytes
   // read by the checked build only: shorter limits of the waits (0: the usual ones), arrivals at the start and
-  // numbers of words (or arrivals) within an attempt that nothing reaches
+  // numbers of words (or arrivals) within an attempt that nothing reaches, and whether the launch is refused
   struct {
-    int start_spins, spins, missing_arrivals, missing_words;
+    int start_spins, spins, missing_arrivals, missing_words, refuse;
   } test;
 };
 

@@ -1,9 +1,9 @@
-"""Resident check periods whose waits run out.
+"""Resident check periods whose waits run out or whose launch is refused.
 
 In the checked build the limits of the waits can be made short, and an arrival
 or a word can be awaited that nothing ever sends (lpop_resident_limits): the
-kernel gives up after the limit, sets its error status and returns.  Nothing
-faults or hangs.
+kernel gives up after the limit, sets its error status and returns.  A refused
+launch is an error code in the place of the call.  Nothing faults or hangs.
 """
 import subprocess
 import sys
@@ -25,6 +25,7 @@ import paper_2506_17650_gb300 as lpop
 lpop.load_library(lib)
 raw = ctypes.CDLL(lib)
 lps = {
+    "one_cta": lambda: lpgen.tiny_random(3),
     "words": lambda: lpgen.batch_member(9, 701, 1_753),
     "barriers": lambda: lpgen.row_length_mix(2),
     "far": lambda: lpgen.powerlaw(2, 50_000, 125_000, 800_000),
@@ -33,7 +34,7 @@ KEYS = ("x", "y", "T", "Sigma", "ax", "xbar", "ybar", "GT", "GS")
 
 
 def limits(p, **k):
-    args = [k.get(n, 0) for n in ("start_spins", "spins", "missing_arrivals", "missing_words")]
+    args = [k.get(n, 0) for n in ("start_spins", "spins", "missing_arrivals", "missing_words", "refuse")]
     assert raw.lpop_resident_limits(p.handle, *args) == 0
 
 
@@ -45,8 +46,9 @@ def error(fn):
     return None
 
 
-lp = lps[case]()
-p = lpop.Problem(lp, alpha=1e-4, phi=7)
+lp = lps[case.split("/")[0]]()
+options = dict(alpha=1e-4, phi=7, precision=case.endswith("/mixed"))
+p = lpop.Problem(lp, **options)
 '''
 
 
@@ -82,3 +84,43 @@ assert st["iterations"] == 64 and np.all(np.isfinite(x)) and np.all(np.isfinite(
 @pytest.mark.parametrize("case", ["words", "barriers", "far"])
 def test_state_lost_in_a_period_is_refused_until_it_is_set_again(case):
     _run(LOST, case)
+
+
+NOT_STARTED = r'''
+p.close()
+more = (dict(), dict(mode=lpop.LP_MODE_PLAIN, scheduler=lpop.LP_SCHED_ADAGRAD_NORM, normalize=0, use_graph=0),
+        dict(scheduler=lpop.LP_SCHED_CONST, restart=0, check_every=16, phi=1))
+for extra in more:
+    opts = dict(options, **extra)
+    with lpop.Problem(lp, **opts) as p, lpop.Problem(lp, **opts) as q:
+        limits(p, **dict(start_spins=500, missing_arrivals=1) if start else dict(refuse=1))
+        for stop in (64, 100, 256):
+            n0 = [x.kernel_times()[2] for x in (p, q)]
+            p.solve(0.0, stop)
+            q.solve(0.0, stop)
+            a, b = p.get_state(), q.get_state()
+            assert all(np.array_equal(a[k], b[k]) for k in KEYS), (extra, stop)
+            assert a["eta"] == b["eta"] and a["k"] == b["k"] and a["attempts"] == stop
+            n1 = [x.kernel_times()[2] for x in (p, q)]
+            assert n1[0] - n0[0] >= 2 * 36 > n1[1] - n0[1]
+'''
+
+
+@pytest.mark.parametrize("start", [True, False])
+@pytest.mark.parametrize("case", ["words", "words/mixed", "barriers", "barriers/mixed", "far"])
+def test_period_that_cannot_be_resident_runs_stepped_with_the_same_bits(case, start):
+    _run(f"start = {start}" + NOT_STARTED, case)
+
+
+ONE_CTA = r'''
+limits(p, refuse=1)
+p.solve(0.0, 40)
+with lpop.Problem(lp, kernel_timing=1, **options) as q:  # timing selects the two step kernels
+    q.solve(0.0, 40)
+    a, b = p.get_state(), q.get_state()
+    assert all(np.array_equal(a[k], b[k]) for k in KEYS)
+'''
+
+
+def test_one_cta_that_is_refused_takes_the_step_kernels():
+    _run(ONE_CTA, "one_cta")
