@@ -98,7 +98,7 @@ struct lp_problem {
     bool ok = false;
     bool alone = true;  // the launch may be resident (false once one was refused or not all of its CTAs started)
     ResPlan plan{};
-    cudaGraphExec_t gexec = nullptr;  // a check period of the plan's stepped launches
+    cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // a check period of the plan's stepped launches (1: in a crowd)
   } res[2];
   // a resident period gave up in the middle of an attempt: its CTAs stopped at different points of the
   // update, so that nothing but a new state (lp_reset, lp_set_state) makes sense
@@ -632,15 +632,15 @@ int create_events(lp_problem* p) {
 bool sampled(const lp_problem* p, int a) { return p->opt.kernel_timing && (a % timing_stride(p)) == 0; }
 
 // One check period as a graph: of the two step kernels or, with a plan, of its stepped launches.
-int capture_graph(lp_problem* p, bool fp32, const ResPlan* plan = nullptr) {
-  cudaGraphExec_t* slot = plan ? &p->res[fp32 ? 1 : 0].gexec : fp32 ? &p->gexec32 : &p->gexec;
+int capture_graph(lp_problem* p, bool fp32, const ResPlan* plan = nullptr, bool crowd = false) {
+  cudaGraphExec_t* slot = plan ? &p->res[fp32 ? 1 : 0].gexec[crowd] : fp32 ? &p->gexec32 : &p->gexec;
   if (*slot) return LP_OK;
   cudaGraph_t g = nullptr;
   CK(cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal));
   const int ce = p->opt.check_every;
   for (int a = 0; a < ce; ++a) {
     if (plan) {
-      launch_stepped(p->d, p->prm, *plan, fp32, p->stream);
+      launch_stepped(p->d, p->prm, *plan, fp32, crowd, p->stream);
       continue;
     }
     const bool tm = sampled(p, a);
@@ -799,7 +799,8 @@ void release(lp_problem* p) {
   if (p->gexec) cudaGraphExecDestroy(p->gexec);
   if (p->gexec32) cudaGraphExecDestroy(p->gexec32);
   for (lp_problem::Resident& R : p->res)
-    if (R.gexec) cudaGraphExecDestroy(R.gexec);
+    for (cudaGraphExec_t g : R.gexec)
+      if (g) cudaGraphExecDestroy(g);
   for (auto e : p->events)
     if (e) cudaEventDestroy(e);
   for (void* v : p->allocs) cudaFree(v);
@@ -1053,16 +1054,18 @@ const ResPlan* resident_plan(lp_problem* p, int* rc) {
 }
 
 // A (part of a) check period in one launch.  *ran: false, with nothing done,
-// where the launch was refused (a context that may use part of the SMs) or not
-// all of its CTAs started within the limit: then the plan's stepped launches
-// take over for good, with the same bits (with one CTA: the two step kernels).
+// where other solves and rounds want the SMs, and for good where the launch was
+// refused (a context that may use part of the SMs) or not all of its CTAs started
+// within the limit: then the plan's stepped launches take over, with the same
+// bits (with one CTA: the two step kernels).
 int run_resident(lp_problem* p, const ResPlan& plan, bool fp32, int nrun, bool check, bool* ran, int* status) {
   lp_problem::Resident& R = p->res[fp32 ? 1 : 0];
   *ran = false;
   if (!R.alone) return LP_OK;
   int fault = 0;
   {
-    SmLease lease(p->device, p->sms, plan.G > 1 ? plan.G : 0, plan.G);
+    ResidentLease lease(p->device, p->sms, plan.G);
+    if (!lease.ok) return LP_OK;
     if (launch_resident(p->d, p->prm, plan, fp32, nrun, p->stream) != cudaSuccess) {
       cudaGetLastError();
       R.alone = false;
@@ -1087,17 +1090,18 @@ int run_resident(lp_problem* p, const ResPlan& plan, bool fp32, int nrun, bool c
   return LP_OK;
 }
 
-// The same in two launches per attempt.
+// The same in plain launches.
 int run_stepped(lp_problem* p, const ResPlan& plan, bool fp32, int nrun, bool check, int* status) {
+  const bool crowd = sm_tokens(p->device, p->sms).crowded();
   if (p->opt.use_graph && nrun == p->opt.check_every) {
-    TRY(capture_graph(p, fp32, &plan));
-    CK(cudaGraphLaunch(p->res[fp32 ? 1 : 0].gexec, p->stream));
+    TRY(capture_graph(p, fp32, &plan, crowd));
+    CK(cudaGraphLaunch(p->res[fp32 ? 1 : 0].gexec[crowd], p->stream));
   } else {
-    for (int a = 0; a < nrun; ++a) launch_stepped(p->d, p->prm, plan, fp32, p->stream);
+    for (int a = 0; a < nrun; ++a) launch_stepped(p->d, p->prm, plan, fp32, crowd, p->stream);
     if (check) launch_check(p->d, p->prm, 0, fp32, p->stream);
     CK(cudaGetLastError());
   }
-  p->launches += 2LL * nrun + (check ? check_kernel_count() : 0);
+  p->launches += (long long)stepped_launches(plan) * nrun + (check ? check_kernel_count() : 0);
   return read_status(p, status);
 }
 
@@ -1120,6 +1124,7 @@ int solve_impl(lp_problem* p, double tol, int64_t iter_limit, int32_t* status_ou
     TRY(maybe_log(p));
   }
   int out_status = LP_STATUS_NONE;
+  SmDemand demand(p->device, p->sms, false);
   while (status == 0 && p->host_attempts < iter_limit) {
     NvtxRange period("lpop check period");
     const bool fp32 = p->fp32_phase;
@@ -1129,6 +1134,7 @@ int solve_impl(lp_problem* p, double tol, int64_t iter_limit, int32_t* status_ou
     int rrc = LP_OK;
     const ResPlan* plan = resident ? resident_plan(p, &rrc) : nullptr;
     TRY(rrc);
+    demand.set(plan && plan->G > 1 ? plan->G : 0);
     if (plan) {
       const long long nrun = to_boundary < remaining ? to_boundary : remaining;
       checked = nrun == to_boundary;

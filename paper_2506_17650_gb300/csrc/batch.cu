@@ -569,6 +569,8 @@ int launch_round(lp_batch* b, const std::vector<int>& active, int attempts) {
   if (rc != LP_OK) return rc;
   const int per_sm = std::max(1, (most + b->sms - 1) / b->sms);
   const int least = (std::min(most, 2 * C) + per_sm - 1) / per_sm;  // a cluster of each kind
+  SmDemand demand(b->device, b->sms, true);
+  demand.set(b->sms);
   SmLease lease(b->device, b->sms, least, std::max(least, (most + per_sm - 1) / per_sm));
   const int total = std::max(1, std::min(most, lease.count * per_sm) / C) * C;
   std::vector<int> h;

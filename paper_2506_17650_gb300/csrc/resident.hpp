@@ -24,24 +24,55 @@ namespace lpop {
 // Up to `attempts` step attempts in one launch (cooperative when G > 1).
 cudaError_t launch_resident(const Dev& d, const Params& prm, const ResPlan& pl, bool fp32, int attempts,
                             cudaStream_t s);
-// One step attempt of the plan in two plain launches, with the same bits (G > 1).
-void launch_stepped(const Dev& d, const Params& prm, const ResPlan& pl, bool fp32, cudaStream_t s);
+// One step attempt of the plan in plain launches, with the same bits (G > 1); crowd: with fewer warps.
+void launch_stepped(const Dev& d, const Params& prm, const ResPlan& pl, bool fp32, bool crowd, cudaStream_t s);
+int stepped_launches(const ResPlan& pl);  // kernels of that
 cudaError_t resident_smem_limit(int device, int* bytes);  // dynamic shared memory a CTA may take
 
 // The SMs of a device (shared by every problem and batch on it).
 SmTokens& sm_tokens(int device, int sms);
 
-// Between `least` and `most` SMs, held for the lifetime of the object (none for least 0).
+// Between `least` and `most` SMs, held for the lifetime of the object.
 struct SmLease {
-  SmTokens* tokens;
+  SmTokens& tokens;
   int count;
   SmLease(int device, int sms, int least, int most)
-      : tokens(least > 0 ? &sm_tokens(device, sms) : nullptr), count(tokens ? tokens->acquire(least, most) : 0) {}
-  ~SmLease() {
-    if (tokens) tokens->release(count);
-  }
+      : tokens(sm_tokens(device, sms)), count(tokens.acquire(least, most)) {}
+  ~SmLease() { tokens.release(count); }
   SmLease(const SmLease&) = delete;
   SmLease& operator=(const SmLease&) = delete;
+};
+
+// The SMs of a resident period, if it may be one (a plan of one CTA needs none).
+struct ResidentLease {
+  SmTokens* tokens;
+  const int count;
+  bool ok = true;
+  ResidentLease(int device, int sms, int ctas) : tokens(ctas > 1 ? &sm_tokens(device, sms) : nullptr), count(ctas) {
+    if (tokens) ok = tokens->acquire_resident(count);
+  }
+  ~ResidentLease() {
+    if (tokens && ok) tokens->release(count);
+  }
+  ResidentLease(const ResidentLease&) = delete;
+  ResidentLease& operator=(const ResidentLease&) = delete;
+};
+
+// What a solve or a batch round in progress takes of the SMs.
+struct SmDemand {
+  SmTokens& tokens;
+  const bool round;
+  int count = 0;
+  SmDemand(int device, int sms, bool batch_round) : tokens(sm_tokens(device, sms)), round(batch_round) {
+    tokens.announce(0, round);
+  }
+  void set(int want) {
+    if (want != count) tokens.announce(want - count, false);
+    count = want;
+  }
+  ~SmDemand() { tokens.withdraw(count, round); }
+  SmDemand(const SmDemand&) = delete;
+  SmDemand& operator=(const SmDemand&) = delete;
 };
 
 }  // namespace lpop

@@ -255,12 +255,9 @@ bool resident_build(const BinTable& binsA, const BinTable& binsAt, long long m, 
       if (r.item.kind == kOwnKind && r.item.len > kResMaxSegs) return false;
     }
   Deal sides[2];  // of A^T, of A
-  int longest = 0;
-  for (const auto& side : {std::make_pair(&binsAt, &head_at), std::make_pair(&binsA, &head_a)}) {
-    const BinTable& bt = *side.first;
-    if (bt.nbins == 0) continue;
-    longest = std::max(longest, bt.bin[0].width == kSell ? bt.bin[0].len : (*side.second)[1] - (*side.second)[0]);
-  }
+  auto longest = [](const BinTable& bt, const std::vector<int>& head) {
+    return bt.nbins == 0 ? 0 : bt.bin[0].width == kSell ? bt.bin[0].len : head[1] - head[0];
+  };
   const int most = std::min(sms, kResMaxCtas);
   // everything in shared memory, or the entries of A read from L2 each time, or those of A^T, or both
   for (int far : {0, 2, 1, 3}) {
@@ -274,7 +271,8 @@ bool resident_build(const BinTable& binsA, const BinTable& binsAt, long long m, 
       ResPlan& pl = out.plan;
       pl = ResPlan{};
       pl.G = G;
-      pl.longest = longest;
+      pl.longest_p = longest(binsAt, head_at);
+      pl.longest_d = longest(binsA, head_a);
       pl.far = far;
       deal(side_items(binsAt, head_at,
                       far & 1 ? far_lanes : short_row_lanes((double)n / G, (double)nnz / (double)n), G > 1),
@@ -292,6 +290,9 @@ bool resident_build(const BinTable& binsA, const BinTable& binsAt, long long m, 
           r = std::max(r, (C.rows + 1) / 2 * 2);
           l = std::max(l, C.nlong);
         }
+        int items = 0;
+        for (const Deal::Cta& C : sides[side].cta) items = std::max(items, C.items);
+        (side ? pl.warps_d : pl.warps_p) = std::min(kResWarps, std::max(4, items));
       }
       for (int g = 0; g < G; ++g) pl.it = std::max(pl.it, sides[0].cta[g].items + sides[1].cta[g].items);
       pl.smem = res_layout(pl, esize).total;
@@ -305,9 +306,7 @@ bool resident_build(const BinTable& binsA, const BinTable& binsAt, long long m, 
   return false;
 }
 
-
-int SmTokens::acquire(int least, int most) {
-  std::unique_lock<std::mutex> lk(mu_);
+int SmTokens::wait_turn(std::unique_lock<std::mutex>& lk, int least, int most) {
   const unsigned long long me = next_++;
   cv_.wait(lk, [&] { return serving_ == me && free_ >= least; });
   const int got = std::min(free_, most);
@@ -317,12 +316,44 @@ int SmTokens::acquire(int least, int most) {
   return got;
 }
 
+int SmTokens::acquire(int least, int most) {
+  std::unique_lock<std::mutex> lk(mu_);
+  return wait_turn(lk, least, most);
+}
+
+bool SmTokens::acquire_resident(int count) {
+  std::unique_lock<std::mutex> lk(mu_);
+  const bool turns = count * kFewSms <= sms_ || wanted_ <= 2 * sms_;
+  if (!turns && wanted_ > sms_) return false;
+  // (a round lasts for many periods: nobody waits for one)
+  if ((next_ != serving_ || free_ < count) && (!turns || rounds_ > 0)) return false;
+  wait_turn(lk, count, count);
+  return true;
+}
+
+bool SmTokens::crowded() {
+  std::lock_guard<std::mutex> lk(mu_);
+  return wanted_ > kCrowd * sms_;
+}
+
 void SmTokens::release(int count) {
   {
     std::lock_guard<std::mutex> lk(mu_);
     free_ += count;
   }
   cv_.notify_all();
+}
+
+void SmTokens::announce(int count, bool round) {
+  std::lock_guard<std::mutex> lk(mu_);
+  wanted_ += count;
+  rounds_ += round;
+}
+
+void SmTokens::withdraw(int count, bool round) {
+  std::lock_guard<std::mutex> lk(mu_);
+  wanted_ -= count;
+  rounds_ -= round;
 }
 
 }  // namespace lpop

@@ -61,8 +61,9 @@ struct ResPlan {
   int ep, ed, rp, rd, lp, ld, it;  // entries, rows, long rows of A^T / A; items of both
   int far;                         // 1: the entries of A^T, 2: those of A are read from the global CSR arrays
   int segs, segs_d;                // segments of both sides, and of A
-  int longest;                     // entries of the longest row of A or A^T
+  int longest_p, longest_d;        // entries of the longest row of A^T and of A
   int smem;                        // dynamic shared memory, bytes
+  int warps_p, warps_d;            // warps of a stepped launch's blocks, for A^T and A
   // read by the checked build only: shorter limits of the waits (0: the usual ones), arrivals at the start and
   // numbers of words (or arrivals) within an attempt that nothing reaches, and whether the launch is refused
   struct {
@@ -128,20 +129,44 @@ int resident_long_rows(const BinTable& bt);  // rows before the first sliced row
 
 // SMs of a device that co-resident kernels hold.  The CTAs of a resident
 // launch wait for one another, so two launches that each got part of the GPU
-// would wait for ever: lp_solve takes the SMs of its launch first, in arrival
-// order, and gives them back when the period has finished; the batched kernel
-// (which would otherwise hold every SM for a whole round) takes what is free.
+// would wait for ever: lp_solve takes the SMs of its launch first and gives them
+// back when the period has finished; the batched kernel (which would otherwise
+// hold every SM for a whole round) takes what is free.
+//
+// One after the other, resident periods leave most of the GPU idle: their
+// attempts are chains of latencies.  Solves from several threads whose plans do
+// not fit side by side therefore run stepped, which gives the same bits and fills
+// the GPU between them; two of them, and small ones, take turns.  us per attempt
+// over all threads, FP64, all in turns / as now (with the two step kernels):
+//   threads                       2                 4                 8                 16
+//   60k nonzeros, 123 CTAs   8.6 / 8.7 (9.7)   8.6 / 4.3 (5.2)   8.7 / 2.9 (3.1)   9.0 / 2.2 (2.4)
+//   linking rows, 152       12.7 /12.7 (14.7) 12.7 / 8.1 (8.4)  12.9 / 5.9 (6.2)  13.2 / 5.3 (6.3)
+//   transport, 152          17.3 /17.9 (18.0) 17.3 /15.6 (16.7) 17.3 /16.6 (16.9) 17.6 /14.4 (17.3)
+//   power law 1e6, 152      32.3 /32.3 (28.1) 31.9 /29.0 (27.6) 31.6 /26.8 (27.5) 32.0 /22.5 (27.6)
+// The stepped blocks have a warp per item, or, with very many solves, one per two.
+constexpr int kFewSms = 8;  // plans of at most this fraction of the SMs take turns
+constexpr int kCrowd = 8;   // very many: plans of this many times the SMs
+
 class SmTokens {
  public:
-  explicit SmTokens(int sms) : free_(sms) {}
+  explicit SmTokens(int sms) : sms_(sms), free_(sms) {}
   // Takes between `least` and `most` SMs, waiting for `least` and for earlier callers.
   int acquire(int least, int most);
+  // Takes `count` SMs for a resident period, or returns false: it should run stepped.
+  bool acquire_resident(int count);
+  bool crowded();
   void release(int count);
+  // SMs that a solve or a batch round in progress takes, or would take by itself.
+  void announce(int count, bool round);
+  void withdraw(int count, bool round);
 
  private:
+  int wait_turn(std::unique_lock<std::mutex>& lk, int least, int most);
   std::mutex mu_;
   std::condition_variable cv_;
+  const int sms_;
   int free_;
+  int wanted_ = 0, rounds_ = 0;
   unsigned long long next_ = 0, serving_ = 0;
 };
 
