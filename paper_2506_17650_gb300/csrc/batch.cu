@@ -487,7 +487,9 @@ int build_schedule(lp_batch* b, const std::vector<int>& active, int total_ctas, 
   for (int id : wide) wide_work += (double)b->nnz[id] + 1.0;
   for (int id : narrow) narrow_work += (double)b->nnz[id] + 1.0;
   int nwide = 0;
-  if (!wide.empty()) {
+  if ((long long)wide.size() + ((long long)narrow.size() + C - 1) / C <= nclusters) {
+    nwide = (int)wide.size();  // a team for every member
+  } else if (!wide.empty()) {
     nwide = (int)std::lround(nclusters * wide_work / (wide_work + narrow_work));
     nwide = std::max(1, std::min(nwide, std::min((int)wide.size(), nclusters - (narrow.empty() ? 0 : 1))));
     if (nwide < 1) nwide = 1;
@@ -567,11 +569,20 @@ int launch_round(lp_batch* b, const std::vector<int>& active, int attempts) {
   int most = 0;
   int rc = resident_ctas(b, cfg, &most);
   if (rc != LP_OK) return rc;
+  // No more than a team for each open member: what a round holds, a solve on
+  // another thread cannot use until it is over.  (Three members of 120k nonzeros,
+  // 256 attempts, 60 ms; beside them 320 attempts of a 60k-nonzero LP: 60 ms with
+  // every SM held, 2.7 so, as alone.)
+  long long wide = 0;
+  for (int id : active) wide += C > 1 && b->nnz[id] >= b->wide_nnz;
+  const long long teams = wide + ((long long)active.size() - wide + C - 1) / C;
+  most = (int)std::min<long long>(most, teams * C);
   const int per_sm = std::max(1, (most + b->sms - 1) / b->sms);
   const int least = (std::min(most, 2 * C) + per_sm - 1) / per_sm;  // a cluster of each kind
+  const int held = std::max(least, (most + per_sm - 1) / per_sm);
   SmDemand demand(b->device, b->sms, true);
-  demand.set(b->sms);
-  SmLease lease(b->device, b->sms, least, std::max(least, (most + per_sm - 1) / per_sm));
+  demand.set(held);
+  SmLease lease(b->device, b->sms, least, held);
   const int total = std::max(1, std::min(most, lease.count * per_sm) / C) * C;
   std::vector<int> h;
   rc = build_schedule(b, active, total, h);
