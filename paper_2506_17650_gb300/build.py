@@ -20,7 +20,8 @@ LIB = os.path.join(HERE, "liblpop.so")
 LIB_CHECKED = os.path.join(HERE, "liblpop_checked.so")
 
 SOURCES = ["api.cu", "kernels_iter.cu", "kernels_check.cu", "kernels_setup.cu", "host_layout.cpp", "device_layout.cu",
-           "noalloc.cu", "batch.cu", "resident.cu", "resident_plan.cpp"]
+           "noalloc.cu", "batch.cu", "resident.cu", "stepped.cu",
+           "resident_plan.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -98,6 +98,7 @@ struct lp_problem {
     bool ok = false;
     bool alone = true;  // the launch may be resident (false once one was refused or not all of its CTAs started)
     ResPlan plan{};
+    StepPlan step{};
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // a check period of the plan's stepped launches (1: in a crowd)
   } res[2];
   // a resident period gave up in the middle of an attempt: its CTAs stopped at different points of the
@@ -640,7 +641,7 @@ int capture_graph(lp_problem* p, bool fp32, const ResPlan* plan = nullptr, bool 
   const int ce = p->opt.check_every;
   for (int a = 0; a < ce; ++a) {
     if (plan) {
-      launch_stepped(p->d, p->prm, *plan, fp32, crowd, p->stream);
+      launch_stepped(p->d, p->prm, *plan, p->res[fp32 ? 1 : 0].step, fp32, crowd, p->stream);
       continue;
     }
     const bool tm = sampled(p, a);
@@ -1044,8 +1045,11 @@ const ResPlan* resident_plan(lp_problem* p, int* rc) {
     h.plan.seg = h.plan.ctl + h.plan.G + 8;
     h.plan.gx = R.block + o3;
     h.plan.bar = reinterpret_cast<unsigned int*>(R.block + o4);
+#ifdef LPOP_CHECK_BOUNDS
     h.plan.test = R.plan.test;
+#endif
     R.plan = h.plan;
+    R.step = h.step;
     R.ok = true;
     return LP_OK;
   };
@@ -1092,16 +1096,17 @@ int run_resident(lp_problem* p, const ResPlan& plan, bool fp32, int nrun, bool c
 
 // The same in plain launches.
 int run_stepped(lp_problem* p, const ResPlan& plan, bool fp32, int nrun, bool check, int* status) {
+  const StepPlan& step = p->res[fp32 ? 1 : 0].step;
   const bool crowd = sm_tokens(p->device, p->sms).crowded();
   if (p->opt.use_graph && nrun == p->opt.check_every) {
     TRY(capture_graph(p, fp32, &plan, crowd));
     CK(cudaGraphLaunch(p->res[fp32 ? 1 : 0].gexec[crowd], p->stream));
   } else {
-    for (int a = 0; a < nrun; ++a) launch_stepped(p->d, p->prm, plan, fp32, crowd, p->stream);
+    for (int a = 0; a < nrun; ++a) launch_stepped(p->d, p->prm, plan, step, fp32, crowd, p->stream);
     if (check) launch_check(p->d, p->prm, 0, fp32, p->stream);
     CK(cudaGetLastError());
   }
-  p->launches += (long long)stepped_launches(plan) * nrun + (check ? check_kernel_count() : 0);
+  p->launches += (long long)stepped_launches(step) * nrun + (check ? check_kernel_count() : 0);
   return read_status(p, status);
 }
 

@@ -25,6 +25,7 @@
 #include <mutex>
 
 #include "ops.cuh"
+#include "resident_sums.cuh"
 
 namespace lpop {
 
@@ -46,117 +47,6 @@ __device__ __forceinline__ constexpr int wait_spins(const ResPlan&) { return kSp
 __device__ __forceinline__ constexpr unsigned int missing_arrivals(const ResPlan&) { return 0u; }
 __device__ __forceinline__ constexpr unsigned int missing_words(const ResPlan&) { return 0u; }
 #endif
-
-// The word of one element of x+ or y+.
-template <class V>
-struct ResElt;
-template <>
-struct ResElt<double> {
-  using T = ulonglong2;
-  static __device__ __forceinline__ void put(T* p, double v, unsigned int seq) {
-    asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }" ::"l"(p),
-                 "l"(__double_as_longlong(v)), "l"((unsigned long long)seq)
-                 : "memory");
-  }
-  // the value, and whether it is of attempt `seq` (or later)
-  static __device__ __forceinline__ bool get(const T* p, unsigned int seq, double* v) {
-    unsigned long long a, b;
-    asm volatile("{ .reg .b128 t; ld.relaxed.gpu.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
-                 : "=l"(a), "=l"(b)
-                 : "l"(p)
-                 : "memory");
-    *v = __longlong_as_double((long long)a);
-    return (int)((unsigned int)b - seq) >= 0;
-  }
-};
-template <>
-struct ResElt<float> {
-  using T = unsigned long long;
-  static __device__ __forceinline__ void put(T* p, float v, unsigned int seq) {
-    const T w = (T)seq << 32 | (T)__float_as_uint(v);
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
-  }
-  static __device__ __forceinline__ bool get(const T* p, unsigned int seq, float* v) {
-    T w;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
-    *v = __uint_as_float((unsigned int)w);
-    return (int)((unsigned int)(w >> 32) - seq) >= 0;
-  }
-};
-
-// What the rows of one side gather: the vector x (one CTA: in shared memory;
-// with barriers: the global vector, by plain loads that the L1 may serve), or
-// the words of the other CTAs of this launch.
-// How a launch's CTAs see one another's x+ and y+.
-enum ResKind { kSoloKind = 0, kWordsKind = 1, kBarriersKind = 2 };
-
-template <class V, int kKind>
-struct ResGather {
-  const V* x;
-  const typename ResElt<V>::T* g;
-  unsigned int seq;
-  int n;
-  unsigned int* bad;
-  int spins;
-  // xv[u] = x[c[u step]] for u < min(4, count); false if a word did not come
-  __device__ __forceinline__ bool four(const int* c, int step, int count, V (&xv)[4]) const {
-    const int none = -1;
-    int j[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      j[u] = u < count ? c[u * step] : none;
-      xv[u] = V(0);
-#ifdef LPOP_CHECK_BOUNDS
-      if (j[u] != none && (unsigned)j[u] >= (unsigned)n) {
-        if (bad) atomicAdd(bad, 1u);
-        j[u] = none;
-      }
-#endif
-    }
-    if constexpr (kKind != kWordsKind) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (j[u] != none) xv[u] = x[j[u]];
-      return true;
-    } else {
-      for (int t = 0; t < spins; ++t) {
-        bool here = true;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (j[u] != none) here = ResElt<V>::get(g + j[u], seq, xv + u) && here;
-        if (here) return true;
-      }
-      return false;
-    }
-  }
-};
-
-// sum over k < count of v[k step] x[c[k step]], four gathers in flight.
-// `most` is the warp's largest count: terms past it are skipped by a uniform
-// branch.  FP64 sums over several CTAs in two chains (a gather's latency is
-// already there, and a chain of 55-65 cycles a term on top of it); one CTA's,
-// bound by the FP64 pipe, and FP32 in one.
-template <class V, int kKind>
-__device__ __forceinline__ V res_dot(const V* v, const int* c, int count, int most, int step,
-                                     const ResGather<V, kKind>& g, bool* ok) {
-  constexpr int kChains = sizeof(V) == 8 && kKind != kSoloKind ? 2 : 1;
-  V a[kChains];
-#pragma unroll
-  for (int q = 0; q < kChains; ++q) a[q] = V(0);
-#pragma unroll 1
-  for (int k0 = 0; k0 < most; k0 += 4) {
-    V xv[4] = {V(0), V(0), V(0), V(0)};
-    if (*ok && !g.four(c, step, count - k0, xv)) *ok = false;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (k0 + u >= most) break;
-      if (k0 + u < count) a[u % kChains] = fma(v[u * step], xv[u], a[u % kChains]);
-    }
-    v += 4 * step;
-    c += 4 * step;
-  }
-  return kChains == 2 ? a[0] + a[kChains - 1] : a[0];
-}
 
 // The same for a row of more than kBlockRowThreshold entries in FP32: pieces of
 // eight terms in FP32, added in FP64, as the step kernels sum such a row.  Only
@@ -184,27 +74,6 @@ __device__ __noinline__ double res_dot_pieces(const float* v, const int* c, int 
     a += (double)p;
   }
   return a;
-}
-
-// The kernel's loop over the attempts is straight-line code that each warp
-// runs once per attempt, so its instruction fetches are on the critical path
-// like every other latency: the pieces below are short loops rather than
-// unrolled code (the same sums unrolled took about twice the cycles).
-
-// Sum over the lanes (valid in every lane).
-__device__ __forceinline__ double lane_sum(double t) {
-#pragma unroll 1
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
-}
-
-// Sum of red[32 k + lane] over the lanes and k < nw (slots past nw are 0).
-__device__ __forceinline__ double res_sum(const double* red, int nw) {
-  red += threadIdx.x & 31;
-  double t = 0.0;
-#pragma unroll 1
-  for (int k = 0; k < nw; k += 4, red += 128) t += (red[0] + red[32]) + (red[64] + red[96]);
-  return lane_sum(t);
 }
 
 __device__ __forceinline__ void bar_arrive(unsigned int* bar) {
@@ -241,18 +110,6 @@ __device__ __forceinline__ bool rec_sum(const ulonglong2* rec, int G, unsigned i
   static_assert(K == 5, "five records a lane");
   *out = lane_sum(((v[0] + v[1]) + (v[2] + v[3])) + v[4]);
   return done;
-}
-
-// The same sum over words that are known to be there.
-__device__ __forceinline__ double sum_words(const ulonglong2* rec, int G) {
-  const int lane = threadIdx.x & 31;
-  double v[kResMaxCtas / 32];
-#pragma unroll
-  for (int q = 0; q < kResMaxCtas / 32; ++q) {
-    const int g = lane + 32 * q;
-    v[q] = g < G ? __longlong_as_double((long long)__ldcg(&rec[g].x)) : 0.0;
-  }
-  return lane_sum(((v[0] + v[1]) + (v[2] + v[3])) + v[4]);
 }
 
 constexpr int kFacs = 64;
@@ -741,215 +598,6 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
   }
 }
 
-// ---- the same attempts in two plain launches each --------------------------------
-//
-// A stepped period does what a resident one does, row for row and sum for sum in
-// the same order, so that the two give the same bits, but its blocks wait for
-// nothing: the plan's CTAs are the blocks of two launches per attempt (A^T y and
-// x+; A x+, y+ and, in the last block to finish, the step control), which read
-// the matrix and the vectors from global memory (L2).  It is what a period runs as when
-// the SMs for a resident one are not to be had.  One solve alone takes 15.6 us per
-// attempt so on the 60k-nonzero LP (resident 8.5), 30 on the transportation LP (17),
-// 57 on the power-law LP of 1M nonzeros (33): chains of loads again, and blocks
-// enough for one wave only.  What counts is several at a time, see SmTokens.
-//
-// A block sums its rows with as many warps as it has items (resident_build), so
-// that several problems share an SM.  Its rows' terms go into the resident
-// kernel's kResThreads slots (row t into slot t mod kResThreads) whatever
-// its threads.  Rows cut into segments: the block that has the row forms all of
-// them, or, with a row of more than kOwnSegs, all blocks do in a launch before.
-constexpr int kOwnSegs = 32;
-LPOP_HD bool segments_apart(int longest) { return longest > kOwnSegs * kResSeg; }
-constexpr int kStepThreads = kResThreads;
-
-// Slots of a block's sums that are ever read: res_sum goes through them 128 at a time.
-LPOP_HD int sum_slots(int rows) { return rows >= kResThreads ? kResThreads : (rows + 127) & ~127; }
-
-// Sum of `size` entries from `beg` on, in the order of a resident segment, into a word.
-template <class V>
-__device__ __forceinline__ void step_segment(const CsrT<V>& M, int beg, int size, const ResGather<V, kBarriersKind>& g,
-                                             ulonglong2* word) {
-  const int lane = threadIdx.x & 31;
-  bool ok = true;
-  const V s = res_dot(M.v + beg + lane, M.ci + beg + lane, (size - lane + 31) >> 5, (size + 31) >> 5, 32, g, &ok);
-  const double w = lane_sum((double)s);
-  if (lane == 0) word->x = (unsigned long long)__double_as_longlong(w);
-}
-
-template <class V, bool kPrimal>
-__global__ void __launch_bounds__(kStepThreads, 2) stepped_segments_kernel(Dev d, ResPlan pl) {
-  pdl_wait();
-  const ResCta C = pl.cta[blockIdx.x];
-  const int first = kPrimal ? C.p0 : C.d0, end = kPrimal ? C.p1 : C.d1;
-  const Vecs<V>& v = vecs<V>(d);
-  const CsrT<V> M = kPrimal ? csr_at<V>(d) : csr_a<V>(d);
-  const int cur = d.st->cur;
-  const ResGather<V, kBarriersKind> g{kPrimal ? v.y[cur] : v.x[cur ^ 1], nullptr, 0u, kPrimal ? d.m : d.n, d.bad_gathers, 0};
-#pragma unroll 1
-  for (int i = first + (int)(threadIdx.x >> 5); i < end; i += (int)(blockDim.x >> 5)) {
-    const ResItem I = pl.items[i];
-    if (I.kind != kSegKind) break;  // (segments come first)
-    step_segment(M, M.rp[I.row0] + I.len, I.nrows, g, pl.seg + I.vec);
-  }
-  pdl_trigger();
-}
-
-template <class V, bool kPrimal>
-__global__ void __launch_bounds__(kStepThreads, 2) stepped_kernel(Dev d, Params prm, ResPlan pl) {
-  constexpr int kAcc = kPrimal ? 3 : 4;
-  extern __shared__ __align__(16) unsigned char s_raw[];
-  __shared__ double s_tot[8];
-  __shared__ double s_fac[2];
-  __shared__ DevState s_st;
-  __shared__ int s_last;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, threads = blockDim.x, warps = threads >> 5;
-  pdl_wait();
-  const ResCta C = pl.cta[blockIdx.x];
-  const ResItem* const it = pl.items + (kPrimal ? C.p0 : C.d0);
-  const int items = kPrimal ? C.p1 - C.p0 : C.d1 - C.d0, rows = kPrimal ? C.rp : C.rd;
-  const int most_rows = kPrimal ? pl.rp : pl.rd, slots = sum_slots(most_rows);
-  double* const s_red = reinterpret_cast<double*>(s_raw);  // kAcc fields of `slots`
-  V* const s_sum = reinterpret_cast<V*>(s_red + kAcc * slots);  // by local row
-  int* const s_row = reinterpret_cast<int*>(s_sum + most_rows);
-  const Vecs<V>& v = vecs<V>(d);
-  const CsrT<V> M = kPrimal ? csr_at<V>(d) : csr_a<V>(d);
-  std::conditional_t<kPrimal, PrimalOp<V, true>, DualOp<V, true>> op;
-  op.sc = read_scalars<V>(d.st, kPrimal);
-  const int cur = op.sc.cur;
-  if constexpr (kPrimal) op.bind(v, prm, cur);
-  else op.bind(v, prm, d.sense, cur);
-  const bool collect = op.sc.collect != 0;
-  const ResGather<V, kBarriersKind> g{kPrimal ? v.y[cur] : v.x[cur ^ 1], nullptr, 0u, kPrimal ? d.m : d.n, d.bad_gathers, 0};
-  bool ok = true;
-  // ---- row sums -----------------------------------------------------------------
-  int own = items;  // the rows cut into segments come last
-  while (own > 0 && it[own - 1].kind == kOwnKind) --own;
-#pragma unroll 1
-  for (int i = warp; i < own; i += warps) {
-    const ResItem I = it[i];
-    if (I.kind == kSegKind) continue;
-    if (lane < I.nrows) s_row[I.vec + lane] = I.row0 + lane;
-    const int width = I.kind == 0 ? 1 : I.kind, lg = 31 - __clz(width);
-    const int l = lane & (width - 1), r = lane >> lg;
-    const bool has = r < I.nrows;
-    const int e0 = has ? M.rp[I.row0 + r] : 0, len = has ? M.rp[I.row0 + r + 1] - e0 : 0;
-    const int count = max(len - l + width - 1, 0) >> lg;
-    const int most = __reduce_max_sync(0xffffffffu, count);
-    V s = res_dot(M.v + e0 + l, M.ci + e0 + l, count, most, width, g, &ok);
-#pragma unroll 1
-    for (int o = width / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, width);
-    if (l == 0 && has) s_sum[I.vec + r] = s;
-  }
-  if (own < items) {
-    int at = 0;  // segments of the rows before
-    const bool apart = segments_apart(kPrimal ? pl.longest_p : pl.longest_d);
-#pragma unroll 1
-    for (int i = own; i < items && !apart; ++i) {
-      const ResItem I = it[i];
-      const int e0 = M.rp[I.row0], e1 = M.rp[I.row0 + 1];
-#pragma unroll 1
-      for (int k = (warp + warps - at) % warps; k < I.len; k += warps)
-        step_segment(M, e0 + k * kResSeg, min(kResSeg, e1 - e0 - k * kResSeg), g, pl.seg + I.ent + k);
-      at = (at + I.len) % warps;
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int i = own + warp; i < items; i += warps) {
-      const ResItem I = it[i];
-      const double t = sum_words(pl.seg + I.ent, I.len);
-      if (lane == 0) {
-        s_sum[I.vec] = (V)t;
-        s_row[I.vec] = I.row0;
-      }
-    }
-  }
-  __syncthreads();
-  // ---- x+ or y+ -------------------------------------------------------------------
-#pragma unroll 1
-  for (int slot = tid; slot < slots; slot += threads) {
-#pragma unroll
-    for (int q = 0; q < kAcc; ++q) op.acc[q] = V(0);
-#pragma unroll 1
-    for (int t = slot; t < rows; t += kResThreads) {
-      const V s[1] = {s_sum[t]};
-      op.prefetch(s_row[t]);
-      op.row(s_row[t], s);
-    }
-#pragma unroll
-    for (int q = 0; q < kAcc; ++q) s_red[q * slots + slot] = (double)op.acc[q];
-  }
-  // ---- this block's record ----------------------------------------------------------
-  __syncthreads();
-  const int fields = collect ? kAcc : kPrimal ? 1 : 2;  // (the others are 0 unless they are recorded)
-  if (warp < fields) {
-    const double t = res_sum(s_red + warp * slots, min(kResWarps, (rows + 31) / 32));
-    if (lane == 0) s_tot[warp] = t;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    const int field[4] = {kPrimal ? 2 : 0, kPrimal ? 5 : 1, kPrimal ? 6 : 3, 4};  // (as in resident_kernel)
-    for (int q = 0; q < fields; ++q)
-      pl.rec[field[q] * pl.G + blockIdx.x].x = (unsigned long long)__double_as_longlong(s_tot[q]);
-    if (!kPrimal) {
-      unsigned int t;
-      asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(t) : "l"(pl.bar + 4) : "memory");
-      s_last = t == gridDim.x - 1;
-    }
-  }
-  if constexpr (kPrimal) {
-    pdl_trigger();
-  } else {
-    __syncthreads();
-    if (!s_last) return;
-    pdl_trigger();
-    // ---- totals and step control ----------------------------------------------------
-    double* const sd = reinterpret_cast<double*>(&s_st);
-    for (int t = tid; t < (int)(sizeof(DevState) / 8); t += threads) sd[t] = reinterpret_cast<const double*>(d.st)[t];
-    for (int f = warp; f < (collect ? 7 : 3); f += warps) {
-      const double t = sum_words(pl.rec + f * pl.G, pl.G);
-      if (lane == 0) s_tot[f] = t;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      step_factors(d.step_tab, s_st.attempts + 1, s_fac, s_fac + 1);
-      const double t1[3] = {s_tot[2], collect ? s_tot[5] : 0.0, collect ? s_tot[6] : 0.0};
-      const double t2[4] = {s_tot[0], s_tot[1], collect ? s_tot[3] : 0.0, collect ? s_tot[4] : 0.0};
-      step_control_state(s_st, prm, s_fac[0], s_fac[1], t1, t2);
-      pl.bar[4] = 0u;
-    }
-    __syncthreads();
-    for (int t = tid; t < (int)(sizeof(DevState) / 8); t += threads) reinterpret_cast<double*>(d.st)[t] = sd[t];
-  }
-}
-
-// (at most 4 x 512 sums, and 5,800 rows of a CTA by 8 bytes or 3,200 by 12)
-constexpr int kSteppedSmem = 56 * 1024;
-
-template <class... KArgs, class... Args>
-void launch_stepped_part(void (*kernel)(KArgs...), int grid, int warps, int smem, cudaStream_t s, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3(32u * (unsigned)warps, 1, 1);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, args...);  // errors surface through cudaGetLastError
-}
-
-template <class V, bool kPrimal>
-void launch_stepped_half(const Dev& d, const Params& prm, const ResPlan& pl, bool crowd, cudaStream_t s) {
-  const int rows = kPrimal ? pl.rp : pl.rd, most = kPrimal ? pl.warps_p : pl.warps_d;
-  const int warps = crowd ? std::max(4, (most + 1) / 2) : most;
-  if (segments_apart(kPrimal ? pl.longest_p : pl.longest_d))
-    launch_stepped_part(stepped_segments_kernel<V, kPrimal>, pl.G, warps, 0, s, d, pl);
-  launch_stepped_part(stepped_kernel<V, kPrimal>, pl.G, warps,
-                      (kPrimal ? 3 : 4) * sum_slots(rows) * 8 + rows * (int)(sizeof(V) + 4), s, d, prm, pl);
-}
-
 template <class V>
 const void* resident_fn_t(int kind) {
   if (kind == kSoloKind) return (const void*)resident_kernel<V, kSoloKind>;
@@ -969,7 +617,7 @@ const void* resident_fn(bool fp32, int kind) {
 constexpr int kWordsMaxRow = 128;
 int resident_kind(const ResPlan& pl) {
   if (pl.G == 1) return kSoloKind;
-  return std::max(pl.longest_p, pl.longest_d) <= kWordsMaxRow && !pl.far ? kWordsKind : kBarriersKind;
+  return pl.longest <= kWordsMaxRow && !pl.far ? kWordsKind : kBarriersKind;
 }
 
 }  // namespace
@@ -990,11 +638,8 @@ cudaError_t resident_smem_limit(int device, int* bytes) {
     if (e != cudaSuccess) return e;
     least = std::min(least, room);
   }
-  for (const void* fn : {(const void*)stepped_kernel<double, true>, (const void*)stepped_kernel<double, false>,
-                         (const void*)stepped_kernel<float, true>, (const void*)stepped_kernel<float, false>}) {
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSteppedSmem);
-    if (e != cudaSuccess) return e;
-  }
+  e = stepped_smem_limit();
+  if (e != cudaSuccess) return e;
   *bytes = least;
   return cudaSuccess;
 }
@@ -1011,20 +656,6 @@ cudaError_t launch_resident(const Dev& d, const Params& prm, const ResPlan& pl, 
   const void* fn = resident_fn(fp32, resident_kind(pl));
   if (pl.G == 1) return cudaLaunchKernel(fn, dim3(1), dim3(kResThreads), args, (size_t)pl.smem, s);
   return cudaLaunchCooperativeKernel(fn, dim3((unsigned)pl.G), dim3(kResThreads), args, (size_t)pl.smem, s);
-}
-
-void launch_stepped(const Dev& d, const Params& prm, const ResPlan& pl, bool fp32, bool crowd, cudaStream_t s) {
-  if (fp32) {
-    launch_stepped_half<float, true>(d, prm, pl, crowd, s);
-    launch_stepped_half<float, false>(d, prm, pl, crowd, s);
-  } else {
-    launch_stepped_half<double, true>(d, prm, pl, crowd, s);
-    launch_stepped_half<double, false>(d, prm, pl, crowd, s);
-  }
-}
-
-int stepped_launches(const ResPlan& pl) {
-  return 2 + segments_apart(pl.longest_p) + segments_apart(pl.longest_d);
 }
 
 SmTokens& sm_tokens(int device, int sms) {

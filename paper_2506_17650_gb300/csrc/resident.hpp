@@ -25,8 +25,10 @@ namespace lpop {
 cudaError_t launch_resident(const Dev& d, const Params& prm, const ResPlan& pl, bool fp32, int attempts,
                             cudaStream_t s);
 // One step attempt of the plan in plain launches, with the same bits (G > 1); crowd: with fewer warps.
-void launch_stepped(const Dev& d, const Params& prm, const ResPlan& pl, bool fp32, bool crowd, cudaStream_t s);
-int stepped_launches(const ResPlan& pl);  // kernels of that
+void launch_stepped(const Dev& d, const Params& prm, const ResPlan& pl, const StepPlan& sp, bool fp32, bool crowd,
+                    cudaStream_t s);
+int stepped_launches(const StepPlan& sp);  // kernels of that
+cudaError_t stepped_smem_limit();  // lets the stepped kernels have the shared memory they may need
 cudaError_t resident_smem_limit(int device, int* bytes);  // dynamic shared memory a CTA may take
 
 // The SMs of a device (shared by every problem and batch on it).

@@ -271,8 +271,9 @@ bool resident_build(const BinTable& binsA, const BinTable& binsAt, long long m, 
       ResPlan& pl = out.plan;
       pl = ResPlan{};
       pl.G = G;
-      pl.longest_p = longest(binsAt, head_at);
-      pl.longest_d = longest(binsA, head_a);
+      out.step.longest[0] = longest(binsAt, head_at);
+      out.step.longest[1] = longest(binsA, head_a);
+      pl.longest = std::max(out.step.longest[0], out.step.longest[1]);
       pl.far = far;
       deal(side_items(binsAt, head_at,
                       far & 1 ? far_lanes : short_row_lanes((double)n / G, (double)nnz / (double)n), G > 1),
@@ -292,7 +293,7 @@ bool resident_build(const BinTable& binsA, const BinTable& binsAt, long long m, 
         }
         int items = 0;
         for (const Deal::Cta& C : sides[side].cta) items = std::max(items, C.items);
-        (side ? pl.warps_d : pl.warps_p) = std::min(kResWarps, std::max(4, items));
+        out.step.warps[side] = std::min(kResWarps, std::max(4, items));
       }
       for (int g = 0; g < G; ++g) pl.it = std::max(pl.it, sides[0].cta[g].items + sides[1].cta[g].items);
       pl.smem = res_layout(pl, esize).total;

@@ -61,14 +61,23 @@ struct ResPlan {
   int ep, ed, rp, rd, lp, ld, it;  // entries, rows, long rows of A^T / A; items of both
   int far;                         // 1: the entries of A^T, 2: those of A are read from the global CSR arrays
   int segs, segs_d;                // segments of both sides, and of A
-  int longest_p, longest_d;        // entries of the longest row of A^T and of A
+  int longest;                     // entries of the longest row of A or A^T
   int smem;                        // dynamic shared memory, bytes
-  int warps_p, warps_d;            // warps of a stepped launch's blocks, for A^T and A
-  // read by the checked build only: shorter limits of the waits (0: the usual ones), arrivals at the start and
-  // numbers of words (or arrivals) within an attempt that nothing reaches, and whether the launch is refused
+#ifdef LPOP_CHECK_BOUNDS
+  // shorter limits of the waits (0: the usual ones), arrivals at the start and numbers of words (or arrivals)
+  // within an attempt that nothing reaches, and whether the launch is refused
   struct {
     int start_spins, spins, missing_arrivals, missing_words, refuse;
   } test;
+#endif
+};
+
+// The same plan's blocks as stepped launches (stepped.cu), for A^T (0) and A (1).  (Not in ResPlan: the compiler
+// lays out the resident kernel anew with the size of its arguments, and with four words more an attempt of the
+// 200,000-variable transportation LP took 17.0 us instead of 16.5.)
+struct StepPlan {
+  int longest[2];  // entries of the longest row
+  int warps[2];    // warps of a block
 };
 
 // Byte offsets of a CTA's arrays in dynamic shared memory.
@@ -116,6 +125,7 @@ struct ResHost {
   std::vector<ResItem> items;
   std::vector<ResCta> cta;
   ResPlan plan{};  // without its device pointers
+  StepPlan step{};
 };
 
 // The plan of a problem's rows (bin tables of A and A^T) for values of
