@@ -1029,6 +1029,7 @@ const ResPlan* resident_plan(lp_problem* p, int* rc) {
     ResHost h;
     if (!resident_build(p->d.binsA, p->d.binsAt, p->d.m, p->d.n, p->nnz, head[0], head[1], esize, p->sms, limit, h))
       return LP_OK;
+    if (p->opt.check_every < shortest_period(h.plan)) return LP_OK;  // (decided by the problem's options: the same path in every call)
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t ib = h.items.size() * sizeof(ResItem), cb = h.cta.size() * sizeof(ResCta);
     const size_t o1 = up(ib), o2 = o1 + up(cb), o3 = o2 + up(16 * (8 * (size_t)h.plan.G + 8 + (size_t)h.plan.segs));
@@ -1058,14 +1059,15 @@ const ResPlan* resident_plan(lp_problem* p, int* rc) {
 }
 
 // A (part of a) check period in one launch.  *ran: false, with nothing done,
-// where other solves and rounds want the SMs, and for good where the launch was
+// where a single attempt is faster stepped (single_attempt_stepped), where other
+// solves and rounds want the SMs, and for good where the launch was
 // refused (a context that may use part of the SMs) or not all of its CTAs started
 // within the limit: then the plan's stepped launches take over, with the same
 // bits (with one CTA: the two step kernels).
 int run_resident(lp_problem* p, const ResPlan& plan, bool fp32, int nrun, bool check, bool* ran, int* status) {
   lp_problem::Resident& R = p->res[fp32 ? 1 : 0];
   *ran = false;
-  if (!R.alone) return LP_OK;
+  if (!R.alone || (nrun == 1 && single_attempt_stepped(plan))) return LP_OK;
   int fault = 0;
   {
     ResidentLease lease(p->device, p->sms, plan.G);

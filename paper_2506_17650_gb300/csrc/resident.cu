@@ -622,6 +622,21 @@ int resident_kind(const ResPlan& pl) {
 
 }  // namespace
 
+// A resident launch loads its rows, forms A^T y once more and writes its rows back,
+// which an attempt or two do not make up for.  us per lp_solve call of one attempt,
+// with the step kernels / resident / stepped: 60k nonzeros 78 / 69 / 65,
+// transportation 92 / 88 / 83, power law 1M (both matrix copies from L2) 114 / 126 /
+// 116; but linking rows 86 / 79 / 81 and power law 100k 83 / 79 / 80.
+bool single_attempt_stepped(const ResPlan& pl) { return pl.G > 1 && (resident_kind(pl) == kWordsKind || pl.far == 3); }
+
+// Shortest check period that resident periods are for.  us per attempt with its
+// checks, step kernels / resident (one attempt a period: stepped where that is
+// the rule above): 1M nonzeros, both copies from L2, a check after every attempt
+// 126 / 136, after every second 84 / 87, every fourth 61 / 58; one CTA, every
+// attempt 64 / 67, every second 41 / 36; others, every attempt: 60k nonzeros 74 / 66,
+// linking rows 88 / 83, transportation 100 / 88, power law 100k 81 / 81.
+int shortest_period(const ResPlan& pl) { return pl.far == 3 ? 4 : pl.G == 1 ? 2 : 1; }
+
 // Dynamic shared memory that a resident CTA may take; also lets the stepped kernels have theirs.
 cudaError_t resident_smem_limit(int device, int* bytes) {
   int optin = 0;

@@ -27,6 +27,8 @@ cudaError_t launch_resident(const Dev& d, const Params& prm, const ResPlan& pl, 
 // One step attempt of the plan in plain launches, with the same bits (G > 1); crowd: with fewer warps.
 void launch_stepped(const Dev& d, const Params& prm, const ResPlan& pl, const StepPlan& sp, bool fp32, bool crowd,
                     cudaStream_t s);
+bool single_attempt_stepped(const ResPlan& pl);  // whether a launch of one attempt had better be stepped
+int shortest_period(const ResPlan& pl);  // check periods below this take the two step kernels
 int stepped_launches(const StepPlan& sp);  // kernels of that
 cudaError_t stepped_smem_limit();  // lets the stepped kernels have the shared memory they may need
 cudaError_t resident_smem_limit(int device, int* bytes);  // dynamic shared memory a CTA may take
