@@ -33,7 +33,8 @@ void launch_begin_solve(DevState* st, double tol, cudaStream_t s);
 // noalloc.cu
 size_t power_norm_state_bytes();
 cudaError_t power_norm(int m, int n, long long nnz, const Csr& A, const Csr& At, int iters, const int* perm,
-                       bool in_order, double* w, double* t, double* part, void* state, cudaStream_t s, double* norm);
+                       const BinTable* binsA, const BinTable* binsAt, double* w, double* t, double* part, void* state,
+                       cudaStream_t s, double* norm);
 void row_kernel_blocks_per_sm(int* primal, int* dual, int* primal32, int* dual32);
 }  // namespace lpop
 
@@ -357,7 +358,7 @@ int preprocess(lp_problem* p) {
     p->norm_est = 0.0;
     if (p->nnz > 0 && p->longest <= kPowerMaxRow) {
       double nw = 0.0;
-      CK(power_norm(m, n, p->nnz, d.A, d.At, p->opt.power_iters, p->d_pcol, true, w, t, red, red + 1024, s, &nw));
+      CK(power_norm(m, n, p->nnz, d.A, d.At, p->opt.power_iters, p->d_pcol, &d.binsA, &d.binsAt, w, t, red, red + 1024, s, &nw));
       p->norm_est = nw > 0.0 && std::isfinite(nw) ? std::sqrt(nw) : 0.0;
     } else if (p->nnz > 0) {
       launch_fill(v, 1.0 / std::sqrt((double)n), n, s);

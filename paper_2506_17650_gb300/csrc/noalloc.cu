@@ -15,6 +15,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "../../include/lpop.h"
 #include "common.cuh"
@@ -82,9 +83,21 @@ __global__ void norm_init_kernel(NormState* st) { *st = NormState{0.0, 1.0, 0.0,
 // for rows of 6 entries spent three quarters of the pipe on lane sums).  Rows
 // of more than 32 W entries wait and are then taken by the whole warp, one by one.
 // 120,000 x 300,000, 1.8M nonzeros, 200 rounds: 13.4 -> 5.5 ms.
-template <int W, bool kNorm>
-__global__ void __launch_bounds__(kBlock) norm_rows_kernel(int rows, const int* rp, const int* ci, const double* v,
-                                                           const double* x, double* y, NormState* st, double* part) {
+//
+// Where the caller has sorted its rows, longest first, the first `wide` take a
+// block each and those up to `head` a warp each, dealt out over the blocks: the
+// longest 32 would otherwise wait for one warp (plain lp_create of a 100k-nonzero
+// power-law LP: 22.7 ms, 6.3 so).
+struct SortedRows {
+  int wide, head;
+};
+struct UnsortedRows {};
+
+template <int W, bool kNorm, class Order>
+__global__ void __launch_bounds__(kBlock, 6) norm_rows_kernel(int rows, const int* rp, const int* ci, const double* v,
+                                                           const double* x, double* y, NormState* st, double* part,
+                                                           Order order) {
+  constexpr bool kSorted = std::is_same<Order, SortedRows>::value;
   __shared__ double smem[kBlock];
   __shared__ int s_last;
   pdl_wait();
@@ -92,31 +105,53 @@ __global__ void __launch_bounds__(kBlock) norm_rows_kernel(int rows, const int* 
   const int warp = (int)(blockIdx.x * kBlock + threadIdx.x) >> 5, warps = (int)(gridDim.x * kBlock) >> 5;
   const double inv = kNorm ? 1.0 : st->inv;
   double acc[1] = {0.0};
-  for (long long r0 = (long long)warp * (32 / W); r0 < rows; r0 += (long long)warps * (32 / W)) {
+  auto dot = [&](int k, int e, int step) {
+    double t = 0.0;
+    for (; k < e; k += 4 * step) {
+      int c[4];
+      double a[4], g[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool ok = k + u * step < e;
+        c[u] = ok ? __ldg(ci + k + u * step) : -1;
+        a[u] = ok ? __ldg(v + k + u * step) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) g[u] = c[u] >= 0 ? __ldg(x + c[u]) : 0.0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (c[u] >= 0) t = fma(a[u], g[u], t);
+    }
+    return t;
+  };
+  if constexpr (kSorted) {
+    for (int row = (int)blockIdx.x; row < order.wide; row += (int)gridDim.x) {
+      double t[1] = {dot(__ldg(rp + row) + (int)threadIdx.x, __ldg(rp + row + 1), kBlock)};
+      block_sum_smem<1>(t, smem);
+      if (threadIdx.x == 0) {
+        y[row] = t[0] * inv;
+        if (kNorm) acc[0] += (t[0] * inv) * (t[0] * inv);
+      }
+    }
+    for (int row = order.wide + (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x; row < order.head; row += warps) {
+      double t = dot(__ldg(rp + row) + lane, __ldg(rp + row + 1), 32);
+      __syncwarp();
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) {
+        y[row] = t * inv;
+        if (kNorm) acc[0] += (t * inv) * (t * inv);
+      }
+    }
+  }
+  int first = 0;
+  if constexpr (kSorted) first = order.head;
+  for (long long r0 = first + (long long)warp * (32 / W); r0 < rows; r0 += (long long)warps * (32 / W)) {
     const long long row = r0 + lane / W;
     const bool has = row < rows;
     const int beg = has ? __ldg(rp + row) : 0, end = has ? __ldg(rp + row + 1) : 0;
     const bool lng = end - beg > 32 * W;
     double s = 0.0;
-    auto dot = [&](int k, int e, int step) {
-      double t = 0.0;
-      for (; k < e; k += 4 * step) {
-        int c[4];
-        double a[4], g[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const bool ok = k + u * step < e;
-          c[u] = ok ? __ldg(ci + k + u * step) : -1;
-          a[u] = ok ? __ldg(v + k + u * step) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) g[u] = c[u] >= 0 ? __ldg(x + c[u]) : 0.0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (c[u] >= 0) t = fma(a[u], g[u], t);
-      }
-      return t;
-    };
     if (!lng) s = dot(beg + sub, end, W);
     __syncwarp();
 #pragma unroll
@@ -163,15 +198,28 @@ __global__ void __launch_bounds__(kBlock) norm_rows_kernel(int rows, const int* 
 
 template <bool kNorm>
 void launch_norm_rows(int rows, const int* rp, const int* ci, const double* val, const double* x, double* y,
-                      NormState* st, double* part, double mean, bool one_lane, cudaStream_t s) {
-  const int W = one_lane && mean <= 16.0 ? 1 : mean <= 8.0 ? 2 : (mean <= 32.0 ? 4 : (mean <= 128.0 ? 8 : 32));
-  const long long warps = ((long long)rows * W + 31) / 32;
-  const int grid = (int)std::min<long long>(912, (warps + kBlock / 32 - 1) / (kBlock / 32));  // six blocks on each of 152 SMs
-  if (W == 1) launch_pdl(norm_rows_kernel<1, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
-  else if (W == 2) launch_pdl(norm_rows_kernel<2, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
-  else if (W == 4) launch_pdl(norm_rows_kernel<4, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
-  else if (W == 8) launch_pdl(norm_rows_kernel<8, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
-  else launch_pdl(norm_rows_kernel<32, kNorm>, grid, s, rows, rp, ci, val, x, y, st, part);
+                      NormState* st, double* part, double mean, const BinTable* sorted, cudaStream_t s) {
+  const int W = sorted && mean <= 16.0 ? 1 : mean <= 8.0 ? 2 : (mean <= 32.0 ? 4 : (mean <= 128.0 ? 8 : 32));
+  // with one lane a row, rows of more than 32 entries by a warp; with 4 or 8, of more than 64 or 256
+  int wide = 0, head = 0;
+  for (int b = 0; sorted && b < sorted->nbins; ++b) {
+    const Bin& B = sorted->bin[b];
+    const bool by_block = B.width == 0 || B.width == kSegmented;
+    if (by_block) wide = B.row_end;
+    if (by_block || (W == 1 && (B.width != kSell || B.len > 32)) || (W == 4 && B.width >= 16) || (W == 8 && B.width == 32))
+      head = B.row_end;
+  }
+  const long long warps = 8LL * wide + (head - wide) + ((long long)(rows - head) * W + 31) / 32;
+  const int grid = (int)std::max<long long>(1, std::min<long long>(912, (warps + kBlock / 32 - 1) / (kBlock / 32)));  // six blocks on each of GB300's 152 SMs
+  auto launch = [&](auto unsorted, auto in_order) {
+    if (sorted) launch_pdl(in_order, grid, s, rows, rp, ci, val, x, y, st, part, SortedRows{wide, head});
+    else launch_pdl(unsorted, grid, s, rows, rp, ci, val, x, y, st, part, UnsortedRows{});
+  };
+  if (W == 1) launch(norm_rows_kernel<2, kNorm, UnsortedRows>, norm_rows_kernel<1, kNorm, SortedRows>);
+  else if (W == 2) launch(norm_rows_kernel<2, kNorm, UnsortedRows>, norm_rows_kernel<2, kNorm, SortedRows>);
+  else if (W == 4) launch(norm_rows_kernel<4, kNorm, UnsortedRows>, norm_rows_kernel<4, kNorm, SortedRows>);
+  else if (W == 8) launch(norm_rows_kernel<8, kNorm, UnsortedRows>, norm_rows_kernel<8, kNorm, SortedRows>);
+  else launch(norm_rows_kernel<32, kNorm, UnsortedRows>, norm_rows_kernel<32, kNorm, SortedRows>);
 }
 
 }  // namespace
@@ -181,11 +229,12 @@ size_t power_norm_state_bytes() { return sizeof(NormState); }
 // ||w|| of the last of `iters` rounds w = A^T A w / ||w|| from the all-ones
 // direction, or (a zero first product: every row of A sums to zero) from the
 // SplitMix64 sign direction.  w [n], t [m], part [1024], state: device scratch.
-// in_order: short rows are summed by one lane, as one chain of FMAs (whether
-// rows that sum to zero give exactly zero depends on that, and with it the
-// start direction).
+// bins: the row classes of A and A^T, whose rows are then sorted, longest first
+// (null: nothing is known of the rows).  With them short rows are summed by one
+// lane, as one chain of FMAs (whether rows that sum to zero give exactly zero
+// depends on that, and with it the start direction).
 cudaError_t power_norm(int m, int n, long long nnz, const Csr& A, const Csr& At, int iters, const int* perm,
-                       bool in_order, double* w, double* t, double* part, void* state, cudaStream_t s, double* norm) {
+                       const BinTable* binsA, const BinTable* binsAt, double* w, double* t, double* part, void* state, cudaStream_t s, double* norm) {
   NormState* st = static_cast<NormState*>(state);
   NormState h{};
   for (int start = 0; start < 2; ++start) {
@@ -198,8 +247,8 @@ cudaError_t power_norm(int m, int n, long long nnz, const Csr& A, const Csr& At,
     }
     norm_init_kernel<<<1, 1, 0, s>>>(st);
     for (int it = 0; it < iters; ++it) {
-      launch_norm_rows<false>(m, A.rp, A.ci, A.v, w, t, st, part, (double)nnz / m, in_order, s);
-      launch_norm_rows<true>(n, At.rp, At.ci, At.v, t, w, st, part, (double)nnz / n, in_order, s);
+      launch_norm_rows<false>(m, A.rp, A.ci, A.v, w, t, st, part, (double)nnz / m, binsA, s);
+      launch_norm_rows<true>(n, At.rp, At.ci, At.v, t, w, st, part, (double)nnz / n, binsAt, s);
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s);
@@ -242,8 +291,8 @@ extern "C" int lp_power_norm_noalloc(int32_t m, int32_t n, const int32_t* a_row_
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   double nw = 0.0;
   if (e == cudaSuccess)
-    e = power_norm(m, n, nnz, Csr{a_row_ptr, a_col_idx, a_val}, Csr{at_row_ptr, at_col_idx, at_val}, iters, nullptr, false,
-                   scratch, scratch + n, scratch + n + m, scratch + kScratchDoubles, s, &nw);
+    e = power_norm(m, n, nnz, Csr{a_row_ptr, a_col_idx, a_val}, Csr{at_row_ptr, at_col_idx, at_val}, iters, nullptr, nullptr,
+                   nullptr, scratch, scratch + n, scratch + n + m, scratch + kScratchDoubles, s, &nw);
   if (e != cudaSuccess) return fail(LP_ERR_CUDA, std::string("power iteration failed: ") + cudaGetErrorString(e));
   *norm_out = nw > 0.0 && std::isfinite(nw) ? std::sqrt(nw) : 0.0;
   return LP_OK;
