@@ -55,22 +55,17 @@ int scratch_address(int dev, double** out) {
   return LP_OK;
 }
 
-// v[j] = scale * (+-1 from SplitMix64 of j, or of perm[j]): the power iteration's second start direction.
-__global__ void splitmix_fill_kernel(double* v, int n, double scale, const int* perm) {
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
-    v[j] = scale * splitmix_sign((unsigned long long)(perm ? perm[j] : j));
-}
-
 // Scalars of the iteration, after the partial sums.
 struct NormState {
   double norm;        // ||w|| of the last round
   double inv;         // what the next product is scaled by: 1 / norm (1 before the first round and for a zero norm)
-  double first;       // ||w|| of the first round
   unsigned int done;  // blocks that have finished in the running launch
   unsigned int rounds;
+  unsigned int restarted;  // the first round's product was zero
+  unsigned int unused;
 };
 
-__global__ void norm_init_kernel(NormState* st) { *st = NormState{0.0, 1.0, 0.0, 0u, 0u}; }
+__global__ void norm_init_kernel(NormState* st) { *st = NormState{0.0, 1.0, 0u, 0u, 0u, 0u}; }
 
 // y = (M x) * st->inv for a CSR matrix whose row lengths nobody has looked at;
 // with kNorm (y = M x then) also ||y|| into the state, by the last block, in a
@@ -88,8 +83,14 @@ __global__ void norm_init_kernel(NormState* st) { *st = NormState{0.0, 1.0, 0.0,
 // block each and those up to `head` a warp each, dealt out over the blocks: the
 // longest 32 would otherwise wait for one warp (plain lp_create of a 100k-nonzero
 // power-law LP: 22.7 ms, 6.3 so).
+//
+// Where the first product is zero, its last warp also writes the second start
+// direction, +-1/sqrt(n) by the SplitMix64 signs of perm[j] (or j): the following
+// launches then go on from there, and the host adds a round (a 60,000 x 20,000
+// incidence matrix, 200 rounds: 4.1 ms with all rounds run twice, 2.1 so).
 struct SortedRows {
   int wide, head;
+  const int* perm;
 };
 struct UnsortedRows {};
 
@@ -187,18 +188,31 @@ __global__ void __launch_bounds__(kBlock, 6) norm_rows_kernel(int rows, const in
   double sum[1] = {0.0};
   for (int b = threadIdx.x; b < (int)gridDim.x; b += kBlock) sum[0] += __ldcg(part + b);
   block_sum_smem<1>(sum, smem);
+  if (threadIdx.x >= 32) return;
+  const bool zero = __double_as_longlong(sum[0]) == 0;  // (the sum is in every lane and not negative)
+  const bool again = zero && st->rounds == 0u;
+  __syncwarp();
   if (threadIdx.x == 0) {
     const double nw = sqrt(sum[0]);
     st->norm = nw;
-    st->inv = nw == 0.0 ? 1.0 : 1.0 / nw;
-    if (st->rounds++ == 0) st->first = nw;
+    st->inv = zero ? 1.0 : 1.0 / nw;
+    st->rounds += 1u;
+    if (again) st->restarted = 1u;
     st->done = 0u;
+  }
+  if (again) {
+    const double one = 1.0 / sqrt((double)rows);
+    for (int j = threadIdx.x; j < rows; j += 32) {
+      int col = j;
+      if constexpr (kSorted) col = order.perm ? order.perm[j] : j;
+      y[j] = one * splitmix_sign((unsigned long long)col);
+    }
   }
 }
 
 template <bool kNorm>
 void launch_norm_rows(int rows, const int* rp, const int* ci, const double* val, const double* x, double* y,
-                      NormState* st, double* part, double mean, const BinTable* sorted, cudaStream_t s) {
+                      NormState* st, double* part, double mean, const BinTable* sorted, const int* perm, cudaStream_t s) {
   const int W = sorted && mean <= 16.0 ? 1 : mean <= 8.0 ? 2 : (mean <= 32.0 ? 4 : (mean <= 128.0 ? 8 : 32));
   // with one lane a row, rows of more than 32 entries by a warp; with 4 or 8, of more than 64 or 256
   int wide = 0, head = 0;
@@ -212,7 +226,7 @@ void launch_norm_rows(int rows, const int* rp, const int* ci, const double* val,
   const long long warps = 8LL * wide + (head - wide) + ((long long)(rows - head) * W + 31) / 32;
   const int grid = (int)std::max<long long>(1, std::min<long long>(912, (warps + kBlock / 32 - 1) / (kBlock / 32)));  // six blocks on each of GB300's 152 SMs
   auto launch = [&](auto unsorted, auto in_order) {
-    if (sorted) launch_pdl(in_order, grid, s, rows, rp, ci, val, x, y, st, part, SortedRows{wide, head});
+    if (sorted) launch_pdl(in_order, grid, s, rows, rp, ci, val, x, y, st, part, SortedRows{wide, head, perm});
     else launch_pdl(unsorted, grid, s, rows, rp, ci, val, x, y, st, part, UnsortedRows{});
   };
   if (W == 1) launch(norm_rows_kernel<2, kNorm, UnsortedRows>, norm_rows_kernel<1, kNorm, SortedRows>);
@@ -236,25 +250,19 @@ size_t power_norm_state_bytes() { return sizeof(NormState); }
 cudaError_t power_norm(int m, int n, long long nnz, const Csr& A, const Csr& At, int iters, const int* perm,
                        const BinTable* binsA, const BinTable* binsAt, double* w, double* t, double* part, void* state, cudaStream_t s, double* norm) {
   NormState* st = static_cast<NormState*>(state);
+  launch_fill(w, 1.0 / std::sqrt((double)n), n, s);
+  norm_init_kernel<<<1, 1, 0, s>>>(st);
   NormState h{};
-  for (int start = 0; start < 2; ++start) {
-    const double one = 1.0 / std::sqrt((double)n);
-    if (start == 0) {
-      launch_fill(w, one, n, s);
-    } else {
-      const int g = (n + kBlock - 1) / kBlock;
-      splitmix_fill_kernel<<<g < 1024 ? g : 1024, kBlock, 0, s>>>(w, n, one, perm);
-    }
-    norm_init_kernel<<<1, 1, 0, s>>>(st);
-    for (int it = 0; it < iters; ++it) {
-      launch_norm_rows<false>(m, A.rp, A.ci, A.v, w, t, st, part, (double)nnz / m, binsA, s);
-      launch_norm_rows<true>(n, At.rp, At.ci, At.v, t, w, st, part, (double)nnz / n, binsAt, s);
+  for (int rounds = iters; rounds > 0;) {
+    for (int it = 0; it < rounds; ++it) {
+      launch_norm_rows<false>(m, A.rp, A.ci, A.v, w, t, st, part, (double)nnz / m, binsA, nullptr, s);
+      launch_norm_rows<true>(n, At.rp, At.ci, At.v, t, w, st, part, (double)nnz / n, binsAt, perm, s);
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
-    if (h.first != 0.0) break;
+    rounds = rounds == iters && h.restarted && h.rounds == (unsigned)iters ? 1 : 0;  // the round that was lost
   }
   *norm = h.norm;
   return cudaSuccess;

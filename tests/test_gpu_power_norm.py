@@ -11,6 +11,7 @@ import scipy.sparse as sp
 
 import lpgen
 import paper_2506_17650_gb300 as lpop
+from oracle.pdhg import splitmix_signs
 from paper_2506_17650_gb300 import build as lpbuild
 
 pytestmark = pytest.mark.gpu
@@ -62,3 +63,30 @@ def test_norm_matches_the_iteration_in_numpy(case, iters):
     got = lpop.lp_power_norm_noalloc(lp.m, lp.n, *[a.data_ptr() for a in arrays], iters=iters,
                                      stream=torch.cuda.current_stream().cuda_stream)
     assert got == pytest.approx(want, rel=1e-11)
+
+
+@pytest.mark.parametrize("iters", [1, 2, 30])
+def test_zero_first_product_starts_again_from_the_signs(iters):
+    """Rows w (x_i - x_k): the all-ones direction gives exactly zero; ``iters`` rounds from the
+    SplitMix64 signs follow, by the caller's column index."""
+    import torch
+
+    rng = np.random.default_rng(0)
+    m, n = 700, 2_000
+    i = rng.integers(0, n, m)
+    k = (i + 1 + rng.integers(0, n - 1, m)) % n
+    w = rng.uniform(0.5, 2.0, m)
+    A = sp.csr_matrix((np.concatenate([w, -w]), (np.tile(np.arange(m), 2), np.concatenate([i, k]))), shape=(m, n))
+    A.sort_indices()
+    v = splitmix_signs(n) / np.sqrt(n)
+    for _ in range(iters):
+        z = A.T @ (A @ v)
+        norm = np.linalg.norm(z)
+        v = z / norm
+    arrays = []
+    for M in (A, A.T.tocsr()):
+        M.sort_indices()
+        arrays += [torch.tensor(a, device="cuda") for a in (M.indptr.astype(np.int32), M.indices.astype(np.int32), M.data)]
+    got = lpop.lp_power_norm_noalloc(m, n, *[a.data_ptr() for a in arrays], iters=iters,
+                                     stream=torch.cuda.current_stream().cuda_stream)
+    assert got == pytest.approx(np.sqrt(norm), rel=1e-11)
