@@ -264,8 +264,8 @@ int lp_kernel_times(lp_problem* p, double* ms, int64_t* samples, int32_t n_kerne
  * cudaMalloc -- code inside a framework that has reserved device memory for
  * its own pool, a real-time loop that must not allocate, or a caller whose
  * buffers come from another allocator -- and that already hold the matrix on
- * the device.  It allocates nothing: its scratch (three work vectors and the
- * reduction's partial sums) is one fixed device array of 2^20 doubles (8 MiB)
+ * the device.  It allocates nothing: its scratch (work vectors, partial sums
+ * and scalars) is one fixed device array of 2^20 doubles (8 MiB)
  * that every GPU which loads this library holds until the process exits.
  *   m, n        rows and columns, m >= 1, n >= 1, and 2 n + m + 1025 <= 2^20
  *               (larger sizes are rejected with LP_ERR_INVALID_ARG)

@@ -552,6 +552,8 @@ int upload(lp_problem* p, int m, int n, long long nz, const int64_t* row_ptr, co
   d.gridAt = grid_of(d.binsAt.nunits, cap_p);
   d.gridA32 = grid_of(d.binsA.nunits, sms * per_sm_d32);
   d.gridAt32 = grid_of(d.binsAt.nunits, sms * per_sm_p32);
+  if (!check_row_classes(d.binsA) || !check_row_classes(d.binsAt))
+    return set_err(p, LP_ERR_CUDA, "the layout has a row class that the kernels do not know");
   for (int which = 0; which < 2; ++which) {
     BinTable& bt = which ? d.binsAt : d.binsA;
     const std::vector<int>& units = which ? segAt : segA;

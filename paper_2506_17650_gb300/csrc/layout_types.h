@@ -119,4 +119,14 @@ struct BinTable {
   const float* sell_v32;
 };
 
+// Whether the row kernels (spmv.cuh) have code for every row of the table: the
+// classes of a layout without widening.
+inline bool check_row_classes(const BinTable& bt) {
+  for (int b = 0; b < bt.nbins; ++b) {
+    const int w = bt.bin[b].width;
+    if (w != 0 && w != kSegmented && w != kSell && w != 4 && w != 16 && w != 32) return false;
+  }
+  return true;
+}
+
 }  // namespace lpop

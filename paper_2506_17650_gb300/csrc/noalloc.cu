@@ -8,8 +8,10 @@
 // caller whose device buffers come from another allocator.  Such a caller
 // already holds its matrix on the device and only wants the estimate.
 //
-// The scratch (three work vectors and the norm reduction's partial sums) lives
-// in one file-scope device array of fixed size, so the call allocates nothing.
+// The scratch (two work vectors, the blocks' partial sums and the iteration's
+// scalars) lives in one file-scope device array of fixed size, so the call
+// allocates nothing.  (Sizes are still refused by the bound of an earlier form
+// with three vectors, 2 n + m + 1025 doubles.)
 // Every GPU that loads the library keeps that array until the process exits.
 #include <algorithm>
 #include <cstring>
@@ -27,7 +29,7 @@ namespace {
 
 // 2^20 doubles = 8 MiB of scratch per device
 constexpr long long kScratchDoubles = 1LL << 20;
-constexpr long long kReduceDoubles = 1 + 1024;  // norm result + per-block partials of launch_norm2
+constexpr long long kReduceDoubles = 1 + 1024;  // per-block partial sums, and one
 
 // (and a few more for the iteration's scalars)
 __device__ __align__(256) double g_noalloc_scratch[kScratchDoubles + 8];
@@ -248,7 +250,8 @@ size_t power_norm_state_bytes() { return sizeof(NormState); }
 // lane, as one chain of FMAs (whether rows that sum to zero give exactly zero
 // depends on that, and with it the start direction).
 cudaError_t power_norm(int m, int n, long long nnz, const Csr& A, const Csr& At, int iters, const int* perm,
-                       const BinTable* binsA, const BinTable* binsAt, double* w, double* t, double* part, void* state, cudaStream_t s, double* norm) {
+                       const BinTable* binsA, const BinTable* binsAt, double* w, double* t, double* part, void* state,
+                       cudaStream_t s, double* norm) {
   NormState* st = static_cast<NormState*>(state);
   launch_fill(w, 1.0 / std::sqrt((double)n), n, s);
   norm_init_kernel<<<1, 1, 0, s>>>(st);

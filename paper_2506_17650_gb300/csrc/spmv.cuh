@@ -73,8 +73,8 @@ struct AllowsPair : std::true_type {};
 template <class Op>
 struct AllowsPair<Op, std::void_t<decltype(Op::kNoPair)>> : std::false_type {};
 
-// Ops of the setup kernels, which also run before the sliced copies are filled
-// (and with 8 lanes per row): those that declare kCsrOnly.
+// Ops of the setup kernels, which also run before the sliced copies are filled:
+// those that declare kCsrOnly.
 template <class Op, class = void>
 struct ReadsCsrOnly : std::false_type {};
 template <class Op>
@@ -358,7 +358,8 @@ __device__ __forceinline__ void wide_unit(const BinTable& bt, int local, int row
 
 // Work units first_unit, first_unit + unit_stride, ... of the table (one block
 // per unit at a time).  smem must hold 32 * NV doubles.  row_slots: see
-// segment_unit.
+// wide_unit.  Rows of other widths than check_row_classes() lets through would be
+// left out.
 template <int NV, class V, class Acc, class G, class Op>
 __device__ __forceinline__ void for_each_row_range(const BinTable& bt, const CsrT<V>& M, const G& g,
                                                    Op& op, double* smem, int first_unit, int unit_stride,
@@ -394,12 +395,11 @@ __device__ __forceinline__ void for_each_row_range(const BinTable& bt, const Csr
 #pragma unroll 1
         for (int r = r0; r < r1; r += kBlock) vec_rows<1, NV, V, Acc>(r, min(r1, r + kBlock), M, g, op);
       }
-    } else {  // the widths a layout gives its rows (and 8, of the no-allocation power iteration)
+    } else {
       const int r0 = B.row_begin + local * (kBlock / width);
       if (width == 4) vec_rows<4, NV, V, Acc>(r0, B.row_end, M, g, op);
       else if (width == 16) vec_rows<16, NV, V, Acc>(r0, B.row_end, M, g, op);
       else if (width == 32) vec_rows<32, NV, V, Acc>(r0, B.row_end, M, g, op);
-      else if constexpr (ReadsCsrOnly<Op>::value) vec_rows<8, NV, V, Acc>(r0, B.row_end, M, g, op);
     }
   }
 }
