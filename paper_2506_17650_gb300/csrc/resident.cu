@@ -320,8 +320,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(Dev d, Params 
     for (int i = warp - w0; i < n; i += kResWarps - w0) {
       const ResItem& I = it[i];
       if (!kSolo && I.kind == kOwnKind) {  // the segments' sums, in segment order over the lanes
-        double t = 0.0;
-        ok = ok && rec_sum(pl.seg + I.ent, I.len, g.seq, g.spins, &t);
+        double t;
+        ok = rec_sum(pl.seg + I.ent, I.len, g.seq, g.spins, &t) && ok;
         if (lane == 0) sum[I.vec] = (V)t;
         continue;
       }
