@@ -452,15 +452,17 @@ int sliced_unit_rows(const BinTable& bt, int cap, int sms) {
   return best;
 }
 
-// The A-row step kernel holds the x of the longest columns (which come first)
-// in shared memory when they have at least a quarter of the entries and every
-// SM has its full blocks.  Entries per block: on the 30M-nonzero power-law LP
-// (about half of all entries are in its 1,024 longest columns) the FP64 kernel
-// took 163.2 us without, 151.6 with 256 to 1,536 and 166.8 with 2,048, the FP32
-// one 129.8 without, 123.5 with 2,048 or 3,072, 113.9 with 4,096 and 117.1 with
-// 5,120.
-constexpr int kHotX = 1024;
-constexpr int kHotX32 = 4096;
+// The FP32 A-row step kernel holds the x of the 4,096 longest columns (which come
+// first) in shared memory when they have at least a quarter of the entries, every
+// SM has its full blocks, and a block gathers at least twice as many entries as
+// it loads there.  us per FP32 attempt without / with it, power-law LPs of
+// exponents 1.8 to 2.3 (the columns have 0.15 to 0.73 of the entries): 3M nonzeros 46-51 /
+// 49-53, 6M 83-90 / 82-89, 12M 132-146 / 131-143, 30M 270-320 / 265-306 (the
+// benchmark's: 305.5 / 287.5); entries per block: 2,048 and 5,120 instead of 4,096
+// cost 123 and 117 us of the kernel's time there, 4,096 114, none 130.  The FP64 kernel
+// has no such variant: with the x of 1,024 columns an attempt took 1-4% longer on
+// every one of them (the benchmark's LP 417.0 / 429.9).
+constexpr int kHotX = 4096;
 
 // Device buffers and the layout: the CSR copies of A and A^T and the vectors
 // in bin order are built on the device from the caller's (valid, canonical)
@@ -566,17 +568,14 @@ int upload(lp_problem* p, int m, int n, long long nz, const int64_t* row_ptr, co
     CK(cudaMemsetAsync(bt.ticket, 0, sizeof(unsigned int) * bt.seg_rows, p->stream));
     bt.seg_unit = su;
   }
-  // x of the longest columns, for the A-row step kernel's gathers
+  // x of the longest columns, for the FP32 A-row step kernel's gathers
   {
-    const int hot = kHotX, hot32 = kHotX32;
-    d.hot = d.hot32 = 0;
-    if (n > hot32 && d.gridA >= cap_d) {
-      int entries[2] = {0, 0};
-      for (int k = 0; k < 2; ++k)
-        CK(cudaMemcpyAsync(entries + k, d.At_rp + (k ? hot32 : hot), sizeof(int), cudaMemcpyDeviceToHost, p->stream));
+    d.hot = 0;
+    if (p->mixed && n > kHotX && d.gridA >= cap_d && nz >= 2LL * kHotX * d.gridA32) {
+      int entries = 0;
+      CK(cudaMemcpyAsync(&entries, d.At_rp + kHotX, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
       CK(cudaStreamSynchronize(p->stream));
-      if (4LL * entries[0] >= nz) d.hot = hot;
-      if (4LL * entries[1] >= nz) d.hot32 = hot32;
+      if (4LL * entries >= nz) d.hot = kHotX;
     }
   }
   p->longest = 2048;

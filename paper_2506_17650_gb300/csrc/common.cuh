@@ -184,7 +184,8 @@ struct Dev {
   unsigned int* bad_gathers;  // checked builds: gathers whose index fell outside the vector
   BinTable binsA, binsAt;
   int gridA, gridAt;      // blocks launched for the A / A^T row kernels (FP64)
-  int hot, hot32;         // first entries of x that a block of the A-row step kernel holds in shared memory (FP64, FP32)
+  int hot;                // first entries of x that a block of the FP32 A-row step kernel holds in shared memory
+  int unused;             // (the resident kernels' code changes with the size of their arguments, see StepPlan)
   int gridA32, gridAt32;  // the same for the FP32 kernels (fewer registers, more resident blocks)
   int max_grid;
 };

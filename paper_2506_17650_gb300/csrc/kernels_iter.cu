@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kBlock, kStepBlocksPerSm<V>) dual_step_kernel(
   g.bad = d.bad_gathers;
   if constexpr (kHot) {
     V* const hot = reinterpret_cast<V*>(s_hot);
-    const int nhot = sizeof(V) == 4 ? d.hot32 : d.hot;
+    const int nhot = d.hot;
     for (int i = threadIdx.x; i < nhot * (int)sizeof(V) / 16; i += kBlock)
       reinterpret_cast<int4*>(hot)[i] = __ldg(reinterpret_cast<const int4*>(v.x[nxt]) + i);
     __syncthreads();
@@ -191,11 +191,10 @@ void launch_primal(const Dev& d, const Params& prm, bool fp32, cudaStream_t s) {
 
 void launch_dual(const Dev& d, const Params& prm, bool fp32, cudaStream_t s) {
   if (fp32) {
-    if (d.hot32 > 0) launch_pdl_smem(dual_step_kernel<float, true>, d.gridA32, d.hot32 * (int)sizeof(float), s, d, prm);
+    if (d.hot > 0) launch_pdl_smem(dual_step_kernel<float, true>, d.gridA32, d.hot * (int)sizeof(float), s, d, prm);
     else launch_pdl(dual_step_kernel<float, false>, d.gridA32, s, d, prm);
   } else {
-    if (d.hot > 0) launch_pdl_smem(dual_step_kernel<double, true>, d.gridA, d.hot * (int)sizeof(double), s, d, prm);
-    else launch_pdl(dual_step_kernel<double, false>, d.gridA, s, d, prm);
+    launch_pdl(dual_step_kernel<double, false>, d.gridA, s, d, prm);
   }
 }
 

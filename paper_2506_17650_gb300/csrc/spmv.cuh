@@ -47,9 +47,9 @@ __device__ __forceinline__ V gather(const Gather<NV, V>& g, int q, int c) {
 
 // A gather whose first nhot entries are in shared memory.  Columns are stored
 // longest first, so with power-law degrees the first few thousand entries of x
-// are about half of all that the rows of A gather; from shared memory a warp's
-// gather takes its bank conflicts (about 7 cycles in FP64) instead of a cycle
-// of the load unit for each lane's line.
+// are a quarter to half of all that the rows of A gather; from shared memory a
+// warp's gather takes its bank conflicts instead of a cycle of the load unit for
+// each lane's line.  (Pays in FP32 only, see kHotX.)
 template <class V>
 struct HotGather : Gather<1, V> {
   const V* hot;

@@ -102,12 +102,12 @@ def test_fp32_step_from_the_oracle_state(case):
 
 
 def test_x_of_the_longest_columns_from_shared_memory():
-    """A power-law LP whose A-row grid is full and whose 1,024 (FP32: 4,096) longest columns have a
-    quarter of the entries: the kernel holds their x in shared memory."""
-    lp = lpgen.powerlaw(3, 130_001, 325_003, 2_000_000)
+    """A power-law LP whose A-row grid is full, whose 4,096 longest columns have a quarter of the
+    entries, and with enough entries per block: the FP32 kernel holds their x in shared memory."""
+    lp = lpgen.powerlaw(3, 360_001, 900_003, 5_600_000)
     o = oracle.Options(alpha=1e-6, phi=2)
     degree = np.sort(np.bincount(lp.col_idx, minlength=lp.n))[::-1]
-    assert 4 * degree[:1024].sum() >= lp.nnz
+    assert 4 * degree[:4096].sum() >= lp.nnz >= 2 * 4096 * 4 * 152  # (four blocks on an SM in FP32)
     P, states = oracle_steps(lp, o, 4)
     for precision, bar in ((lpop.LP_PREC_FP64, 1e-12), (lpop.LP_PREC_MIXED, 1e-5)):
         with lpop.Problem(lp, **gpu_options(o, kernel_timing=1, precision=precision)) as p:
