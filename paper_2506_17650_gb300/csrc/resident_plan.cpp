@@ -220,6 +220,16 @@ constexpr long long kResSmem = 220 * 1024;  // what a CTA's rows may take, rough
 // 2,439 -> 2,004 (four lanes 2,197); 1.4M, both sides, 2,608 -> 3,076, so not.
 constexpr int kFarLanes = 4, kFarLanesBoth = 2;
 constexpr long long kFarBothMax = 1 << 20;
+// (FP64, 0.6M to 1.04M entries of five families, 27 LPs: 0.49 to 0.99 of the step kernels' time.)
+
+// Shared memory of a CTA up to which one side may be read from L2 when there are
+// more entries than that: above it the next size of the shared memory leaves 28 KB of
+// the SM's 256 for the L1, which serves the gathers and what several lanes read
+// of a sector.  us per attempt, step kernels / one side far: FP64 1.3M entries (187 KB
+// of shared memory) 31.1 / 26.0, 1.4M (205 KB) 31.1 / 34.0, 1.5M (215 KB) 32.0 / 35.6;
+// FP32 1.4M (191 KB) 31.9 / 25.5, 1.5M (205 KB) 32.8 / 35.6, linking rows 1.8M (189 KB)
+// 36.6 / 29.6, 1.96M (203 KB) 38.5 / 40.9.
+constexpr int kFarSmem = 193 * 1024;  // of 196 KB, with the kernel's static share and the system's
 
 // Cycles of the FP64 pipe per attempt and CTA that a problem is split down to
 // (600 to 2,000 measured the same within 2%: the chain of latencies between the
@@ -297,7 +307,7 @@ bool resident_build(const BinTable& binsA, const BinTable& binsAt, long long m, 
       }
       for (int g = 0; g < G; ++g) pl.it = std::max(pl.it, sides[0].cta[g].items + sides[1].cta[g].items);
       pl.smem = res_layout(pl, esize).total;
-      if (pl.smem <= smem_limit) {
+      if (pl.smem <= (far && nnz > kFarBothMax ? std::min(smem_limit, kFarSmem) : smem_limit)) {
         lay_out(sides, out);
         return true;
       }

@@ -62,17 +62,17 @@ def test_both_copies_far():
         assert _close(got[0][key], got[1][key]), f"{key} against the step kernels"
 
 
-@pytest.mark.parametrize("size", [(100_000, 250_000, 1_500_000), (160_000, 400_000, 1_040_000), (50_000, 125_000, 800_000)])
+@pytest.mark.parametrize("size", [(86_666, 216_666, 1_300_000), (160_000, 400_000, 1_040_000), (50_000, 125_000, 800_000)])
 def test_fp32_attempts_match_the_step_kernels(size):
     lp = lpgen.powerlaw(2, *size)
     o = dict(alpha=1e-4, phi=5, precision=lpop.LP_PREC_MIXED)
     with lpop.Problem(lp, kernel_timing=1, **o) as step, lpop.Problem(lp, **o) as p:
-        for k in (1, 2, 6, 7, 20, 63):
+        for k in (1, 4, 7, 20, 63):
             step.solve(0.0, k - 1)
             p.set_state(step.get_state())
             n0 = p.kernel_times()[2]
             p.solve(0.0, k + 1)  # two attempts: a resident launch (one alone may run stepped)
-            assert p.kernel_times()[2] <= n0 + 2 * CHECK + 2
+            assert p.kernel_times()[2] == n0 + 1 + CHECK
             step.solve(0.0, k + 1)
             a, b = p.get_state(), step.get_state()
             for key in ("x", "y", "T", "Sigma", "ax", "xbar", "ybar"):
