@@ -101,15 +101,18 @@ typedef struct lp_options {
   double precond_floor;      /* projection floor for T and Sigma; default 1e-6 */
   int32_t ruiz_iters;        /* Ruiz rounds (Section 2); default 10 */
   double pc_beta;            /* Pock-Chambolle exponent beta in [0, 2] (pdlp mode); default 1 */
-  int32_t check_every;       /* attempts between KKT / restart checks, 1..65536 (one check period is
-                                captured as one CUDA graph); default 64 */
+  int32_t check_every;       /* attempts between KKT / restart checks, 1..65536; default 64.  (Very short
+                                periods take other kernels, whose sums differ in the last bits.) */
   int32_t restart;           /* adaptive restarts in pdlp mode; default 1 */
   int32_t power_iters;       /* power iterations for ||A~||_2 (plain mode); default 200 */
   double plain_step_factor;  /* plain mode step = factor / ||A~||_2; default 0.9 */
   double time_limit;         /* seconds per lp_solve call; <= 0 means none; default 0 */
-  int32_t use_graph;         /* replay one check period as a CUDA graph; default 1 */
-  int32_t kernel_timing;     /* time sampled launches of the hot kernels with CUDA events: 0 off (default),
-                                1 one attempt in 8, k >= 2 one attempt in k of each check period */
+  int32_t use_graph;         /* replay a check period of plain launches as a CUDA graph (problems that fit on
+                                the SMs run a period in one launch instead); default 1 */
+  int32_t kernel_timing;     /* time sampled launches of the two step kernels with CUDA events: 0 off (default),
+                                1 one attempt in 8, k >= 2 one attempt in k of each check period.  Timing makes
+                                every problem take the step kernels, also one that would otherwise run its
+                                periods in one launch: other speed, and other last bits of the sums */
   int32_t device;            /* CUDA device ordinal; -1 = the calling thread's current device */
   void* stream;              /* cudaStream_t every launch and copy goes to; NULL = default stream */
   int32_t precision;         /* LP_PREC_*; default LP_PREC_FP64 */

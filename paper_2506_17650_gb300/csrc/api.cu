@@ -2,10 +2,11 @@
 //
 // lp_create validates on the host, copies the caller's arrays to the device
 // once, builds the bin-ordered CSR copies of A and A^T there and runs the
-// preprocessing kernels.  lp_solve drives the
-// device-resident iteration: one check period (check_every step attempts and
-// the KKT check) is captured once as a CUDA graph and replayed; the host only
-// reads one status word per period.
+// preprocessing kernels.  lp_solve drives the device-resident iteration by check
+// periods (check_every step attempts and the KKT check) and reads one status
+// word per period: problems that fit on the SMs run a period's attempts in one
+// resident launch, or stepped (resident.cu, stepped.cu); larger ones replay a
+// period of the two step kernels, captured once as a CUDA graph.
 #include <algorithm>
 #include <chrono>
 #include <cmath>

@@ -613,7 +613,10 @@ const void* resident_fn(bool fp32, int kind) {
 // (the 376k-nonzero LP with rows of up to 3,000 entries: 1,660 us with words,
 // 1,112 with barriers; the other way the 60k-nonzero LP, rows of up to 35
 // entries: 709 us with words, 779 with barriers, the transportation LP 1,293
-// against 1,348).
+// against 1,348).  The line could lie higher for LPs with few long rows: 60k and
+// 300k nonzeros with one row in 200 of 140 / 200 / 400 entries, 657 / 670 / 700 and
+// 772 / 802 / 822 us with words, 723 / 732 / 748 and 844 / 843 / 870 with barriers
+// (the step kernels: 1,290 and 1,470).
 constexpr int kWordsMaxRow = 128;
 int resident_kind(const ResPlan& pl) {
   if (pl.G == 1) return kSoloKind;

@@ -7,13 +7,17 @@
 // GPU waits, and a step control with cold instruction caches.  A problem whose
 // matrix copies and vectors fit in the shared memory of the GPU's SMs is
 // instead split by rows over G CTAs (one per SM) that hold their rows of
-// A and A^T, the rows' vectors and the solver state for a whole check period:
-// per attempt only x+ and y+ travel (through L2), between grid-wide barriers,
-// and every CTA sums the G records and runs the step control on its own copy
-// of the state.  A problem that fits in one SM takes a single CTA and no grid
-// barrier.  Where the vectors fit but not both copies of the matrix, one or both
-// copies are read from global memory (L2) in each attempt.  resident.cu and
-// resident_plan.cpp have the measured times and the choices.
+// A and A^T, the rows' vectors and the solver state for a whole check period.
+// Per attempt only x+ and y+ travel (through L2), as words of a value and the
+// number of its attempt or, with rows that many others gather, between grid-wide
+// barriers; CTA 0 sums the CTAs' records, runs the step control and sends its
+// result to the others.  A problem that fits in one SM takes a single CTA and
+// exchanges nothing.  Where the vectors fit but not both copies of the matrix, one
+// or both copies are read from global memory (L2) in each attempt.  resident.cu
+// and resident_plan.cpp have the measured times and the choices.
+//
+// The same plan can run stepped (stepped.cu): plain launches with the same bits,
+// for periods that cannot have the SMs to themselves.
 #pragma once
 
 #include "common.cuh"
