@@ -187,18 +187,18 @@ __global__ void __launch_bounds__(kBlock, 6) norm_rows_kernel(int rows, const in
   __syncthreads();
   if (!s_last) return;
   pdl_trigger();
+  const unsigned int rounds = st->rounds;
   double sum[1] = {0.0};
   for (int b = threadIdx.x; b < (int)gridDim.x; b += kBlock) sum[0] += __ldcg(part + b);
   block_sum_smem<1>(sum, smem);
   if (threadIdx.x >= 32) return;
   const bool zero = __double_as_longlong(sum[0]) == 0;  // (the sum is in every lane and not negative)
-  const bool again = zero && st->rounds == 0u;
-  __syncwarp();
+  const bool again = zero && rounds == 0u;
   if (threadIdx.x == 0) {
     const double nw = sqrt(sum[0]);
     st->norm = nw;
     st->inv = zero ? 1.0 : 1.0 / nw;
-    st->rounds += 1u;
+    st->rounds = rounds + 1u;
     if (again) st->restarted = 1u;
     st->done = 0u;
   }
