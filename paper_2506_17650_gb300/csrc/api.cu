@@ -1103,8 +1103,12 @@ int run_resident(lp_problem* p, const ResPlan& plan, bool fp32, int nrun, bool c
 int run_stepped(lp_problem* p, const ResPlan& plan, bool fp32, int nrun, bool check, int* status) {
   const StepPlan& step = p->res[fp32 ? 1 : 0].step;
   const bool crowd = sm_tokens(p->device, p->sms).crowded();
-  if (p->opt.use_graph && nrun == p->opt.check_every) {
-    TRY(capture_graph(p, fp32, &plan, crowd));
+  bool graph = p->opt.use_graph && nrun == p->opt.check_every;
+  if (graph && capture_graph(p, fp32, &plan, crowd) != LP_OK) {  // (a stream that cannot be captured)
+    cudaGetLastError();
+    graph = false;
+  }
+  if (graph) {
     CK(cudaGraphLaunch(p->res[fp32 ? 1 : 0].gexec[crowd], p->stream));
   } else {
     for (int a = 0; a < nrun; ++a) launch_stepped(p->d, p->prm, plan, step, fp32, crowd, p->stream);

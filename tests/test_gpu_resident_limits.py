@@ -124,3 +124,17 @@ with lpop.Problem(lp, kernel_timing=1, **options) as q:  # timing selects the tw
 
 def test_one_cta_that_is_refused_takes_the_step_kernels():
     _run(ONE_CTA, "one_cta")
+
+
+LEGACY_STREAM = r'''
+with lpop.Problem(lp, stream=1, **options) as q:  # the legacy default stream, which cannot be captured
+    limits(q, refuse=1)
+    q.solve(0.0, 128)
+    p.solve(0.0, 128)
+    a, b = q.get_state(), p.get_state()
+    assert all(np.array_equal(a[k], b[k]) for k in KEYS)
+'''
+
+
+def test_stepped_period_on_a_stream_that_cannot_be_captured():
+    _run(LEGACY_STREAM, "words")
