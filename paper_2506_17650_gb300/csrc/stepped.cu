@@ -91,7 +91,11 @@ __global__ void __launch_bounds__(kStepThreads, 2) stepped_kernel(Dev d, Params 
   bool ok = true;
   // ---- row sums -----------------------------------------------------------------
   int own = items;  // the rows cut into segments come last
-  while (own > 0 && it[own - 1].kind == kOwnKind) --own;
+  for (int c = 32; c == 32; own -= c) {
+    const int i = own - 1 - lane;
+    const unsigned int rest = __ballot_sync(0xffffffffu, i < 0 || it[i].kind != kOwnKind);
+    c = rest ? __ffs((int)rest) - 1 : 32;
+  }
 #pragma unroll 1
   for (int i = warp; i < own; i += warps) {
     const ResItem I = it[i];
