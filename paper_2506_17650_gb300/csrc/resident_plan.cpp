@@ -219,7 +219,10 @@ constexpr long long kResSmem = 220 * 1024;  // what a CTA's rows may take, rough
 // one side, 2,150 -> 1,527 us (two lanes 1,575, eight 1,690); 1.0M, both sides,
 // 2,439 -> 2,004 (four lanes 2,197); 1.4M, both sides, 2,608 -> 3,076, so not.
 constexpr int kFarLanes = 4, kFarLanesBoth = 2;
-constexpr long long kFarBothMax = 1 << 20;
+// So both may be while a copy's entries take 12 MB: 1,048,576 in FP64, 1,572,864 in
+// FP32 (1.5M, step kernels / both sides far: power law 37.0 / 33.1, random 32.5 / 30.1
+// us per attempt).
+constexpr long long kFarBothBytes = 12LL << 20;
 // (FP64, 0.6M to 1.04M entries of five families, 27 LPs: 0.49 to 0.99 of the step kernels' time.)
 
 // Shared memory of a CTA up to which one side may be read from L2 when there are
@@ -228,7 +231,8 @@ constexpr long long kFarBothMax = 1 << 20;
 // of a sector.  us per attempt, step kernels / one side far: FP64 1.3M entries (187 KB
 // of shared memory) 31.1 / 26.0, 1.4M (205 KB) 31.1 / 34.0, 1.5M (215 KB) 32.0 / 35.6;
 // FP32 1.4M (191 KB) 31.9 / 25.5, 1.5M (205 KB) 32.8 / 35.6, linking rows 1.8M (189 KB)
-// 36.6 / 29.6, 1.96M (203 KB) 38.5 / 40.9.
+// 36.6 / 29.6, 1.96M (203 KB) 38.5 / 40.9.  (Fewer entries: never slower.)
+constexpr long long kFarSmemEntries = 1 << 20;
 constexpr int kFarSmem = 193 * 1024;  // of 196 KB, with the kernel's static share and the system's
 
 // Cycles of the FP64 pipe per attempt and CTA that a problem is split down to
@@ -275,7 +279,12 @@ bool resident_build(const BinTable& binsA, const BinTable& binsAt, long long m, 
     int G = (int)std::min<double>(most, std::max(16.0 * cost / kTargetCycles, (double)foot / (double)kResSmem));
     if (G < 1 || (!far && foot + 48 * 1024 <= (long long)smem_limit)) G = 1;  // (retried with more CTAs if it does not fit after all)
     if (far) G = most;
-    if (foot > (long long)most * smem_limit || (far == 3 && nnz > kFarBothMax)) continue;  // (no need to deal the rows out)
+    if (far == 3 && nnz * (esize + 4) > kFarBothBytes) continue;
+    const int limit = far && nnz > kFarSmemEntries ? std::min(smem_limit, kFarSmem) : smem_limit;
+    // what the CTAs' arrays hold at least (res_layout): no need to deal the rows out when that does not fit
+    const long long least = (far == 3 ? 0 : far ? 1 : 2) * nnz * (esize + 4) + esize * (10 * n + 8 * m) + 5 * n + 6 * m +
+                            9 * ((far & 1 ? n : 0) + (far & 2 ? m : 0)) + (long long)most * 4 * kResThreads * 8;
+    if (least > (long long)most * limit) continue;
     const int far_lanes = far == 3 ? kFarLanesBoth : kFarLanes;
     for (;; G = std::min(most, G + std::max(1, G / 8))) {
       ResPlan& pl = out.plan;
@@ -307,7 +316,7 @@ bool resident_build(const BinTable& binsA, const BinTable& binsAt, long long m, 
       }
       for (int g = 0; g < G; ++g) pl.it = std::max(pl.it, sides[0].cta[g].items + sides[1].cta[g].items);
       pl.smem = res_layout(pl, esize).total;
-      if (pl.smem <= (far && nnz > kFarBothMax ? std::min(smem_limit, kFarSmem) : smem_limit)) {
+      if (pl.smem <= limit) {
         lay_out(sides, out);
         return true;
       }

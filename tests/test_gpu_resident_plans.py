@@ -62,7 +62,7 @@ def test_both_copies_far():
         assert _close(got[0][key], got[1][key]), f"{key} against the step kernels"
 
 
-@pytest.mark.parametrize("size", [(86_666, 216_666, 1_300_000), (160_000, 400_000, 1_040_000), (50_000, 125_000, 800_000)])
+@pytest.mark.parametrize("size", [(86_666, 216_666, 1_300_000), (100_000, 250_000, 1_500_000), (160_000, 400_000, 1_040_000), (50_000, 125_000, 800_000)])
 def test_fp32_attempts_match_the_step_kernels(size):
     lp = lpgen.powerlaw(2, *size)
     o = dict(alpha=1e-4, phi=5, precision=lpop.LP_PREC_MIXED)

@@ -17,11 +17,12 @@ def test_larger_matrices_are_refused_rather_than_read_from_global_memory(runner,
     assert not plan(runner, tmp_path, lpgen.powerlaw(2, 100_000, 250_000, 1_500_000), 8, 152)["ok"]
 
 
-@pytest.mark.parametrize("size,fits", [((86_666, 216_666, 1_300_000), True), ((100_000, 250_000, 1_500_000), False)])
-def test_one_side_far_leaves_room_for_the_l1_beyond_a_million_entries(runner, tmp_path, size, fits):  # noqa: F811
+@pytest.mark.parametrize("size,far", [((86_666, 216_666, 1_300_000), (1, 2)), ((100_000, 250_000, 1_500_000), (3,)),
+                                      ((115_000, 285_000, 1_750_000), ())])
+def test_far_sides_leave_room_for_the_l1_beyond_a_million_entries(runner, tmp_path, size, far):  # noqa: F811
     lp = lpgen.powerlaw(2, *size)
     p = plan(runner, tmp_path, lp, 4, 152)
-    assert bool(p["ok"]) == fits
-    if fits:
-        assert p["far"] in (1, 2) and p["smem"] <= 193 * 1024
+    assert bool(p["ok"]) == bool(far)
+    if far:
+        assert p["far"] in far and p["smem"] <= 193 * 1024
         check(p, lp, "far", 152, 4)
