@@ -226,7 +226,8 @@ void launch_norm_rows(int rows, const int* rp, const int* ci, const double* val,
       head = B.row_end;
   }
   const long long warps = 8LL * wide + (head - wide) + ((long long)(rows - head) * W + 31) / 32;
-  const int grid = (int)std::max<long long>(1, std::min<long long>(912, (warps + kBlock / 32 - 1) / (kBlock / 32)));  // six blocks on each of GB300's 152 SMs
+  constexpr long long kMostBlocks = 912;  // six on each of GB300's 152 SMs
+  const int grid = (int)std::max<long long>(1, std::min(kMostBlocks, (warps + kBlock / 32 - 1) / (kBlock / 32)));
   auto launch = [&](auto unsorted, auto in_order) {
     if (sorted) launch_pdl(in_order, grid, s, rows, rp, ci, val, x, y, st, part, SortedRows{wide, head, perm});
     else launch_pdl(unsorted, grid, s, rows, rp, ci, val, x, y, st, part, UnsortedRows{});
